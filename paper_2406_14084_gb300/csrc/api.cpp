@@ -68,7 +68,10 @@ struct DevPlanBuf {
     void *coef = nullptr;
     void *coef_df = nullptr;  // complex128 plans in double-float form: (h, l) of re, then of im
     int device = -1;
+    bool borrowed = false;    // base is a state's plan_ws, not the plan's own
 };
+
+constexpr size_t kPlanWsMax = size_t(8) << 20;  // larger plans get their own allocation
 
 }  // namespace
 
@@ -82,6 +85,10 @@ struct qs_state {
     std::vector<int> phys_of;  // logical -> physical
     double *scratch = nullptr;
     size_t scratch_bytes = 0;
+    // device memory for the plans that live within one call (qs_apply_circuit, remaps): such a call
+    // ends with a synchronize of the stream, so the next one may overwrite it
+    void *plan_ws = nullptr;
+    size_t plan_ws_bytes = 0;
     qs_stats_t stats{};
     // profiling: event pairs recorded around launches, folded into stats on qs_stats()
     bool profiling = false;
@@ -145,7 +152,7 @@ struct qs_plan {
     ~qs_plan()
     {
         for (auto &d : dev)
-            if (d.base) cudaFree(d.base);
+            if (d.base && !d.borrowed) cudaFree(d.base);
     }
 };
 
@@ -176,14 +183,15 @@ qs_status ensure_scratch(qs_state *s, size_t bytes)
     return QS_OK;
 }
 
-qs_status upload(qs_plan *pl, qs_dtype dt)
+// borrow: put the plan into this state's plan_ws (the caller synchronises before it returns)
+qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
 {
     DevPlanBuf &d = pl->dev[dt];
     int dev = 0;
     cudaGetDevice(&dev);
     if (d.base && d.device == dev) return QS_OK;
     if (d.base) {
-        cudaFree(d.base);
+        if (!d.borrowed) cudaFree(d.base);
         d.base = nullptr;
     }
     const Plan &p = pl->p;
@@ -234,12 +242,39 @@ qs_status upload(qs_plan *pl, qs_dtype dt)
     }
     if (fault("alloc")) return fail(QS_ENOMEM, "injected allocation failure");
     void *base = nullptr;
-    qs_status st = cuda_status(cudaMalloc(&base, total), "plan upload allocation");
-    if (st) return st;
-    st = cuda_status(cudaMemcpy(base, h.data(), total, cudaMemcpyHostToDevice), "plan upload");
-    if (st) {
-        cudaFree(base);
-        return st;
+    qs_status st = QS_OK;
+    d.borrowed = borrow != nullptr && total <= kPlanWsMax;
+    if (d.borrowed) {
+        // a copy recorded into a graph would read the host buffer after it is gone
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        d.borrowed = cudaStreamIsCapturing(borrow->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    }
+    if (d.borrowed) {
+        if (borrow->plan_ws_bytes < total) {
+            if (borrow->plan_ws) {
+                cudaStreamSynchronize(borrow->stream);
+                cudaFree(borrow->plan_ws);
+                borrow->plan_ws = nullptr;
+                borrow->plan_ws_bytes = 0;
+            }
+            st = cuda_status(cudaMalloc(&borrow->plan_ws, total), "plan upload allocation");
+            if (st) {
+                borrow->plan_ws = nullptr;
+                return st;
+            }
+            borrow->plan_ws_bytes = total;
+        }
+        base = borrow->plan_ws;
+        st = cuda_status(cudaMemcpyAsync(base, h.data(), total, cudaMemcpyHostToDevice, borrow->stream), "plan upload");
+        if (st) return st;
+    } else {
+        st = cuda_status(cudaMalloc(&base, total), "plan upload allocation");
+        if (st) return st;
+        st = cuda_status(cudaMemcpy(base, h.data(), total, cudaMemcpyHostToDevice), "plan upload");
+        if (st) {
+            cudaFree(base);
+            return st;
+        }
     }
     d.base = base;
     d.device = dev;
@@ -287,10 +322,11 @@ struct StepTimer {
     }
 };
 
-qs_status run_plan(qs_state *s, qs_plan *pl, StepTimer *timer = nullptr)
+// transient: the plan lives within the caller's call (see upload)
+qs_status run_plan(qs_state *s, qs_plan *pl, StepTimer *timer = nullptr, bool transient = false)
 {
     if (fault("launch")) return fail(QS_ECUDA, "injected launch failure");
-    qs_status st = upload(pl, s->dt);
+    qs_status st = upload(pl, s->dt, transient ? s : nullptr);
     if (st) return st;
     const DevPlanBuf &d = pl->dev[s->dt];
     const Plan &p = pl->p;
@@ -352,10 +388,10 @@ qs_status canonicalize_state(qs_state *s)
     pl->p.n = s->n;
     pl->p.dt = s->dt;
     plan_canonicalize(s->n, s->dt, s->phys_of, pl->p);
-    qs_status st = run_plan(s, pl.get());
-    if (st) return st;
-    // plan buffers are freed by the destructor; wait so the free cannot race the kernels
+    qs_status st = run_plan(s, pl.get(), nullptr, true);
+    // wait: the plan's device memory is reused or freed after this call
     cudaStreamSynchronize(s->stream);
+    if (st) return st;
     for (int q = 0; q < s->n; ++q) s->phys_of[q] = q;
     return QS_OK;
 }
@@ -482,6 +518,7 @@ qs_status qs_destroy(qs_state *s)
     cudaStreamSynchronize(s->stream);
     if (s->owned && s->amp) cudaFree(s->amp);
     if (s->scratch) cudaFree(s->scratch);
+    if (s->plan_ws) cudaFree(s->plan_ws);
     delete s;
     return QS_OK;
     QS_GUARD_END
@@ -861,9 +898,8 @@ qs_status qs_plan_dump(const qs_plan *pl, char *buf, size_t cap, size_t *needed)
     QS_GUARD_END
 }
 
-qs_status qs_apply_plan(qs_state *s, const qs_plan *p)
+static qs_status apply_plan(qs_state *s, const qs_plan *p, bool transient)
 {
-    QS_GUARD_BEGIN
     if (!s || !p) return fail(QS_EINVAL, "NULL argument");
     if (p->p.n != s->n) return fail(QS_EINVAL, "plan and state have different qubit counts");
     if (p->p.dt != s->dt) return fail(QS_EINVAL, "plan was built for the other precision (options.dtype)");
@@ -877,7 +913,7 @@ qs_status qs_apply_plan(qs_state *s, const qs_plan *p)
         // the judge: time this plan on its first apply and the greedy twin on the second
         qs_plan *run = pl->judge_state == 0 ? pl : pl->alt.get();
         StepTimer timer;
-        st = run_plan(s, run, &timer);
+        st = run_plan(s, run, &timer, transient);
         if (st) return st;
         st = cuda_status(cudaEventSynchronize(timer.ev.back()), "judge timing");
         if (st) return st;
@@ -887,10 +923,16 @@ qs_status qs_apply_plan(qs_state *s, const qs_plan *p)
         return QS_OK;
     }
     qs_plan *run = (pl->alt && pl->use_alt) ? pl->alt.get() : pl;
-    st = run_plan(s, run);
+    st = run_plan(s, run, nullptr, transient);
     if (st) return st;
     s->phys_of = run->p.final_phys_of;
     return QS_OK;
+}
+
+qs_status qs_apply_plan(qs_state *s, const qs_plan *p)
+{
+    QS_GUARD_BEGIN
+    return apply_plan(s, p, false);
     QS_GUARD_END
 }
 
@@ -942,9 +984,9 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *g, size_t ng, const qs_op
     qs_plan *p = nullptr;
     qs_status st = qs_fuse(g, ng, s->n, &opt, &p);
     if (st) return st;
-    st = qs_apply_plan(s, p);
+    std::unique_ptr<qs_plan> own(p);
+    st = apply_plan(s, p, true);
     cudaStreamSynchronize(s->stream);
-    delete p;
     return st;
     QS_GUARD_END
 }
@@ -960,9 +1002,9 @@ qs_status qs_remap(qs_state *s, int k, const int *A, const int *B)
     std::string err;
     int rc = plan_remap(s->n, s->dt, a, b, pl->p, err);
     if (rc) return fail((qs_status)rc, err);
-    qs_status st = run_plan(s, pl.get());
-    if (st) return st;
+    qs_status st = run_plan(s, pl.get(), nullptr, true);
     cudaStreamSynchronize(s->stream);
+    if (st) return st;
     std::vector<int> logi(s->n);
     for (int q = 0; q < s->n; ++q) logi[s->phys_of[q]] = q;
     for (int j = 0; j < k; ++j) std::swap(logi[a[j]], logi[b[j]]);

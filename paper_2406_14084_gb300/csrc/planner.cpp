@@ -21,7 +21,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
+#include <memory>
 #include <set>
 
 namespace qs {
@@ -78,15 +78,6 @@ int expected_nt(int kind)
     case QS_UNITARY: case QS_DIAG: return -1;
     default: return 1;
     }
-}
-
-char role_of(const CGate &g, int q)
-{
-    // 'N' = non-diagonal action on q; 'D' = diagonal action (controls, diagonal gates)
-    if (g.cls == C_DIAG) return 'D';
-    for (int t : g.tq)
-        if (t == q) return 'N';
-    return 'D';
 }
 
 std::vector<int> all_qubits(const CGate &g)
@@ -340,32 +331,67 @@ int default_seg_bits(qs_dtype dt) { return dt == QS_C64 ? 4 : 3; }
 
 namespace {
 
-bool hoistable(const CGate &g, const std::map<int, char> &skipped)
+// Qubits a gate touches, and those it acts on non-diagonally, as bit masks.
+struct Roles {
+    uint64_t any = 0, nondiag = 0;
+};
+
+Roles roles_of(const CGate &g)
 {
-    for (int q : all_qubits(g)) {
-        auto it = skipped.find(q);
-        if (it == skipped.end()) continue;
-        if (it->second == 'N' || role_of(g, q) == 'N') return false;
-    }
-    return true;
+    Roles r;
+    for (int q : g.tq) r.any |= 1ull << q;
+    if (g.cls != C_DIAG) r.nondiag = r.any;
+    for (int q : g.cq) r.any |= 1ull << q;
+    return r;
 }
 
-void note_skipped(const CGate &g, std::map<int, char> &skipped)
+// A gate may move ahead of the skipped ones if it meets none of them on a qubit where either acts
+// non-diagonally.
+bool hoistable(const Roles &g, const Roles &skipped)
 {
-    for (int q : all_qubits(g)) {
-        const char r = role_of(g, q);
-        auto it = skipped.find(q);
-        if (it == skipped.end()) skipped[q] = r;
-        else if (r == 'N') it->second = 'N';
-    }
+    return !(g.nondiag & skipped.any) && !(g.any & skipped.nondiag);
+}
+
+void note_skipped(const Roles &g, Roles &skipped)
+{
+    skipped.any |= g.any;
+    skipped.nondiag |= g.nondiag;
+}
+
+// Entry of a diagonal gate (controls folded in) at the basis state whose set qubits are `x`.
+cd diag_entry(const CGate &g, uint64_t x)
+{
+    for (int c : g.cq)
+        if (!(x >> c & 1)) return cd(1.0);
+    size_t l = 0;
+    for (size_t j = 0; j < g.tq.size(); ++j) l |= size_t((x >> g.tq[j]) & 1) << j;
+    return g.m[l];
+}
+
+// Cost of a diagonal that is no controlled phase, over m qubits (the last case of op_cost).
+double table_cost(int m, qs_dtype dt)
+{
+    const double w = dt == QS_C64 ? 1.0 : 62.0, smem = dt == QS_C64 ? 16.0 : 32.0;
+    return m <= 7 ? w * 4.0 + 3.0 : w * 4.0 + 3.0 * m + smem + 2.0;
 }
 
 // Merge g (applied after cur) into cur if allowed.  Returns true on success.
-bool try_merge(CGate &cur, const CGate &g, int kdiag, int kdense, bool force_dense, qs_dtype dt)
+// The costs decide before any matrix product is formed, where they do not depend on it (a planner's
+// time went into products and qubit lists of merges that were then refused).
+bool try_merge(CGate &cur, const CGate &g, const Roles &rc, const Roles &rg, int kdiag, int kdense, bool force_dense,
+               qs_dtype dt)
 {
-    std::vector<int> U = union_qubits(cur, g);
+    const int nu = popcount(rc.any | rg.any);
     if (cur.cls == C_DIAG && g.cls == C_DIAG) {
-        if ((int)U.size() > kdiag) return false;
+        if (nu > kdiag) return false;
+        const double parts = op_cost(cur, dt) + op_cost(g, dt) + 1e-9;
+        if (!force_dense && table_cost(nu, dt) > parts) {
+            // refused unless the product is a controlled phase: every entry but the last is 1.
+            // Entries at no qubit set, and at either gate's own qubits, usually tell.
+            for (uint64_t x : {uint64_t(0), rc.any, rg.any})
+                if (x != (rc.any | rg.any) && diag_entry(cur, x) * diag_entry(g, x) != cd(1.0)) return false;
+        }
+        std::vector<int> U = union_qubits(cur, g);
         std::vector<cd> a = embed_diag(cur, U), b = embed_diag(g, U);
         for (size_t i = 0; i < a.size(); ++i) a[i] *= b[i];
         CGate m;
@@ -373,20 +399,26 @@ bool try_merge(CGate &cur, const CGate &g, int kdiag, int kdense, bool force_den
         m.tq = U;
         m.m = std::move(a);
         m.nsrc = cur.nsrc + g.nsrc;
-        if (!force_dense && op_cost(m, dt) > op_cost(cur, dt) + op_cost(g, dt) + 1e-9) return false;
+        if (!force_dense && op_cost(m, dt) > parts) return false;
         cur = std::move(m);
         return true;
     }
-    if (kdense < 1 || (int)U.size() > kdense) return false;
+    if (kdense < 1 || nu > kdense) return false;
     // dense merge: matrix over U (controls become qubits of the fused gate)
     CGate m;
     m.cls = C_DENSE;
+    if (!force_dense && nu > 1) {
+        // keep controls as controls where possible: a merged op is only worth it if cheaper (the
+        // cost of a matrix on two or more qubits does not depend on its entries)
+        m.tq.resize(nu);
+        if (op_cost(m, dt) > op_cost(cur, dt) + op_cost(g, dt) + 1e-9) return false;
+    }
+    std::vector<int> U = union_qubits(cur, g);
     m.tq = U;
     const size_t D = size_t(1) << U.size();
     m.m = matmul(embed(g, U), embed(cur, U), D);
     m.nsrc = cur.nsrc + g.nsrc;
-    if (!force_dense) {
-        // keep controls as controls where possible: a merged op is only worth it if cheaper
+    if (!force_dense && nu == 1) {
         if (op_cost(m, dt) > op_cost(cur, dt) + op_cost(g, dt) + 1e-9) return false;
     }
     cur = std::move(m);
@@ -399,6 +431,9 @@ std::vector<CGate> fuse_pass(const std::vector<CGate> &in, int kdiag, int kdense
     const int window = 256;
     std::vector<CGate> out;
     std::vector<char> used(in.size(), 0);
+    std::vector<Roles> roles(in.size());
+    for (size_t i = 0; i < in.size(); ++i) roles[i] = roles_of(in[i]);
+    out.reserve(in.size());
     for (size_t i = 0; i < in.size(); ++i) {
         if (used[i]) continue;
         used[i] = 1;
@@ -407,25 +442,21 @@ std::vector<CGate> fuse_pass(const std::vector<CGate> &in, int kdiag, int kdense
             out.push_back(std::move(cur));
             continue;
         }
-        std::map<int, char> skipped;
+        Roles rc = roles[i], skipped;
         for (size_t j = i + 1; j < in.size() && j < i + window; ++j) {
             if (used[j]) continue;
             const CGate &g = in[j];
             bool merged = false;
-            if (hoistable(g, skipped) && !(diag_only && g.cls != C_DIAG))
-                merged = try_merge(cur, g, kdiag, diag_only ? 0 : kdense, force_dense, dt);
+            if (hoistable(roles[j], skipped) && !(diag_only && g.cls != C_DIAG))
+                merged = try_merge(cur, g, rc, roles[j], kdiag, diag_only ? 0 : kdense, force_dense, dt);
             if (merged) {
                 used[j] = 1;
+                rc = roles_of(cur);
                 continue;
             }
-            note_skipped(g, skipped);
+            note_skipped(roles[j], skipped);
             // stop once every qubit of cur is blocked by a non-diagonal skipped gate
-            bool all_blocked = true;
-            for (int q : all_qubits(cur)) {
-                auto it = skipped.find(q);
-                if (it == skipped.end() || it->second != 'N') { all_blocked = false; break; }
-            }
-            if (all_blocked) break;
+            if (!(rc.any & ~skipped.nondiag)) break;
         }
         // a fused product that came out as the identity (H then H, RZ then RZ^-1, ...) does
         // nothing: drop it (a uniform phase is kept, it is not the identity)
@@ -522,7 +553,7 @@ DevOp make_op(const CGate &g, const std::vector<int> &phys, const int *local_of,
 
 struct Sched {
     int gate;
-    std::vector<int> phys;  // logical -> physical snapshot
+    std::shared_ptr<const std::vector<int>> at;  // logical -> physical snapshot, shared while unchanged
 };
 
 // The kernel's XOR swizzle of slab-local indices in shared memory (same map as the device's
@@ -842,7 +873,7 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
     std::vector<char> regable(ns, 0), done(ns, 0);
     for (size_t i = 0; i < ns; ++i) {
         const CGate &g = gates[sched[i].gate];
-        const std::vector<int> &ph = sched[i].phys;
+        const std::vector<int> &ph = *sched[i].at;
         for (int t : g.tq) {
             const int l = local_of[ph[t]];
             if (g.cls == C_DIAG) {
@@ -871,7 +902,7 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
         while (first < ns && done[first]) ++first;
         if (first >= ns) break;
         if (!regable[first]) {
-            plan.ops.push_back(make_op(gates[sched[first].gate], sched[first].phys, local_of, cf));
+            plan.ops.push_back(make_op(gates[sched[first].gate], *sched[first].at, local_of, cf));
             done[first] = 1;
             continue;
         }
@@ -926,7 +957,7 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
         st.sub_begin = (int)plan.subs.size();
         for (size_t j : sub) {
             const CGate &g = gates[sched[j].gate];
-            const std::vector<int> &ph = sched[j].phys;
+            const std::vector<int> &ph = *sched[j].at;
             DevSub s;
             std::memset(&s, 0, sizeof s);
             auto classify = [&](int q) {
@@ -1027,18 +1058,17 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
     }
 }
 
-void emit_pass(Plan &plan, const std::vector<CGate> &gates, std::vector<int> S, int lo, int b, int n,
+void emit_pass(Plan &plan, const std::vector<CGate> &gates, uint64_t S, int lo, int b, int n,
                const std::vector<Sched> &sched, StepKind kind, qs_dtype dt)
 {
     // pad the slab up to b bits with the lowest unused positions
-    std::set<int> inS(S.begin(), S.end());
-    for (int p = 0; (int)inS.size() < b && p < n; ++p) inS.insert(p);
+    for (int p = 0; popcount(S) < b && p < n; ++p) S |= 1ull << p;
     DevPass P;
     std::memset(&P, 0, sizeof P);
     std::vector<int> hi;
-    for (int p : inS)
-        if (p >= lo) hi.push_back(p);
-    P.b = (int)inS.size();
+    for (int p = lo; p < 64; ++p)
+        if (S >> p & 1) hi.push_back(p);
+    P.b = popcount(S);
     P.lo = lo;
     P.nhi = (int)hi.size();
     for (size_t j = 0; j < hi.size(); ++j) P.hipos[j] = (uint8_t)hi[j];
@@ -1489,6 +1519,8 @@ int build_plan(const std::vector<CGate> &gates_in, int n, qs_dtype dt, const qs_
     }
 
     std::vector<char> done(gates.size(), 0);
+    std::vector<Roles> roles(gates.size());
+    for (size_t i = 0; i < gates.size(); ++i) roles[i] = roles_of(gates[i]);
     size_t first = 0;
     int stalls = 0;
     while (true) {
@@ -1501,45 +1533,46 @@ int build_plan(const std::vector<CGate> &gates_in, int n, qs_dtype dt, const qs_
             stalls = 0;
             continue;
         }
-        std::set<int> S;
-        for (int p = 0; p < (lowblock ? b : lo); ++p) S.insert(p);
-        std::map<int, char> skipped;
+        uint64_t S = (1ull << (lowblock ? b : lo)) - 1;  // physical positions in the slab
+        Roles skipped;
+        std::shared_ptr<const std::vector<int>> snapshot;
         std::vector<Sched> sched;
         std::vector<int> wanted;  // low-block mode: logical qubits needed but not resident
         for (size_t i = first; i < gates.size(); ++i) {
             if (done[i]) continue;
             const CGate &g = gates[i];
-            if (!hoistable(g, skipped) || is_tc[i]) {
-                note_skipped(g, skipped);
+            if (!hoistable(roles[i], skipped) || is_tc[i]) {
+                note_skipped(roles[i], skipped);
                 continue;
             }
             if (is_relabel(g)) {
                 const int a = g.tq[0], c = g.tq[1];
+                snapshot.reset();
                 std::swap(phys[a], phys[c]);
                 logi[phys[a]] = a;
                 logi[phys[c]] = c;
                 done[i] = 1;
                 continue;
             }
-            std::vector<int> need;
+            uint64_t want = 0;
             if (g.cls != C_DIAG)
-                for (int t : g.tq)
-                    if (!S.count(phys[t])) need.push_back(phys[t]);
-            const bool fits = lowblock ? need.empty() : (int)(S.size() + need.size()) <= b;
+                for (int t : g.tq) want |= 1ull << phys[t];
+            const bool fits = lowblock ? !(want & ~S) : popcount(S | want) <= b;
             if (fits) {
-                for (int p : need) S.insert(p);
-                sched.push_back({(int)i, phys});
+                S |= want;
+                if (!snapshot) snapshot = std::make_shared<const std::vector<int>>(phys);
+                sched.push_back({(int)i, snapshot});
                 done[i] = 1;
             } else {
                 if (lowblock)
-                    for (int p : need)
-                        if (std::find(wanted.begin(), wanted.end(), logi[p]) == wanted.end())
+                    for (int t : g.tq)
+                        if (const int p = phys[t]; !(S >> p & 1) && std::find(wanted.begin(), wanted.end(), logi[p]) == wanted.end())
                             wanted.push_back(logi[p]);
-                note_skipped(g, skipped);
+                note_skipped(roles[i], skipped);
             }
         }
         if (!sched.empty()) {
-            emit_pass(plan, gates, std::vector<int>(S.begin(), S.end()), lo, b, n, sched, S_PASS, dt);
+            emit_pass(plan, gates, S, lo, b, n, sched, S_PASS, dt);
             stalls = 0;
         }
         while (first < gates.size() && done[first]) ++first;

@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 import numpy as np
@@ -208,29 +209,45 @@ def _check(rc: int):
 
 # ----------------------------------------------------------------------------- marshalling
 
+_PACK_GATE = struct.Struct("<18i3dQ").pack_into  # QsGate: kind, nt, nc, t[7], c[8], p[3], m
+_GATE_BYTES = ctypes.sizeof(QsGate)
+assert _GATE_BYTES == struct.calcsize("<18i3dQ")
+
+
+def _fill_gate(s, g, tg, ct):
+    """Field by field: what the packed form does not take (integers beyond 32 bits)."""
+    s.kind = KINDS[g.kind]
+    s.nt, s.nc = len(tg), len(ct)
+    for j, q in enumerate(tg):
+        s.t[j] = q
+    for j, q in enumerate(ct):
+        s.c[j] = q
+    p = list(g.params) + [0.0] * (3 - len(g.params))
+    for j in range(3):
+        s.p[j] = float(p[j])
+
+
 def marshal_gates(gates):
     arr = (QsGate * max(1, len(gates)))()
     keep = []
     for i, g in enumerate(gates):
-        s = arr[i]
-        s.kind = KINDS[g.kind]
-        tg, ct = list(g.targets), list(g.controls)
-        if not (1 <= len(tg) <= MAX_TARGETS) or len(ct) > MAX_CONTROLS:
+        kind = KINDS[g.kind]
+        tg, ct = tuple(g.targets), tuple(g.controls)
+        nt, nc = len(tg), len(ct)
+        if not (1 <= nt <= MAX_TARGETS) or nc > MAX_CONTROLS:
             raise ValueError(f"gate {i}: bad qubit counts")
-        s.nt, s.nc = len(tg), len(ct)
-        for j, q in enumerate(tg):
-            s.t[j] = q
-        for j, q in enumerate(ct):
-            s.c[j] = q
-        p = list(g.params) + [0.0] * (3 - len(g.params))
-        for j in range(3):
-            s.p[j] = float(p[j])
+        p = tuple(map(float, list(g.params)[:3]))
+        ptr = 0
         if g.matrix is not None:
             m = np.ascontiguousarray(np.asarray(g.matrix, dtype=np.complex128))
             keep.append(m)
-            s.m = m.ctypes.data_as(_dp)
-        else:
-            s.m = _dp()
+            ptr = m.ctypes.data
+        try:
+            _PACK_GATE(arr, i * _GATE_BYTES, kind, nt, nc, *tg, *(0,) * (MAX_TARGETS - nt), *ct,
+                       *(0,) * (MAX_CONTROLS - nc), *p, *(0.0,) * (3 - len(p)), ptr)
+        except struct.error:
+            _fill_gate(arr[i], g, tg, ct)
+            arr[i].m = ctypes.cast(_vp(ptr), _dp)
     return arr, keep
 
 
