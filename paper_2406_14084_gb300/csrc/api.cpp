@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "learned.h"
+#include "lower.h"
 #include "model.h"
 #include "planner.h"
 #include "qs_internal.h"
@@ -67,6 +68,13 @@ struct DevPlanBuf {
     unsigned char *images = nullptr;
     void *coef = nullptr;
     void *coef_df = nullptr;  // complex128 plans in double-float form: (h, l) of re, then of im
+    void *words = nullptr;    // lowered stages and their conditional tables
+    void *pool = nullptr;
+    std::vector<unsigned char> h_words;
+    struct Lean {             // per pass; nstages = 0: some op needs the general kernel
+        int begin = 0, words = 0, stages = 0;
+    };
+    std::vector<Lean> lean;
     int device = -1;
     bool borrowed = false;    // base is a state's plan_ws, not the plan's own
 };
@@ -195,35 +203,66 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
         d.base = nullptr;
     }
     const Plan &p = pl->p;
-    const size_t np = std::max<size_t>(1, p.passes.size()), no = std::max<size_t>(1, p.ops.size());
-    const size_t nc = std::max<size_t>(1, p.coef.size());
-    const size_t nst = std::max<size_t>(1, p.stages.size()), nsb = std::max<size_t>(1, p.subs.size());
-    auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-    const size_t o_pass = 0, o_ops = al(np * sizeof(DevPass));
-    const size_t o_st = o_ops + al(no * sizeof(DevOp)), o_sb = o_st + al(nst * sizeof(DevStage));
-    const size_t ntc = std::max<size_t>(1, p.tcs.size()), nim = std::max<size_t>(16, p.tc_images.size());
-    const size_t o_tc = o_sb + al(nsb * sizeof(DevSub)), o_im = o_tc + al(ntc * sizeof(DevTc));
-    const size_t o_coef = o_im + al(nim);
-    // two spare entries: the register stages read a sub-op's first two coefficients ahead
     const bool want_df = dt == QS_C128 && p.opt.arith == QS_ARITH_DF;
-    const size_t o_cdf = o_coef + al((nc + 2) * amp_bytes(dt));
-    const size_t total = o_cdf + (want_df ? al((nc + 2) * 16) : 0);
+    std::vector<DevStage> stages = p.stages;
+    LeanImage img;
+    lower_stages(p, dt, want_df, stages, img);
+    // The coefficient pool of the general engine is uploaded where some step needs it.
+    d.lean.assign(p.passes.size(), DevPlanBuf::Lean{});
+    bool general = false;
+    for (size_t i = 0; i < p.passes.size(); ++i) {
+        const DevPass &P = p.passes[i];
+        bool lean = !P.has_perm && P.op_begin < P.op_end;
+        for (int o = P.op_begin; lean && o < P.op_end; ++o)
+            lean = p.ops[o].type == OP_STAGE && stages[p.ops[o].mat].lean_begin >= 0;
+        if (lean) {  // the stages of a pass, and so their words, are consecutive
+            const DevStage &s0 = stages[p.ops[P.op_begin].mat], &s1 = stages[p.ops[P.op_end - 1].mat];
+            d.lean[i].begin = s0.lean_begin;
+            d.lean[i].words = s1.lean_begin + s1.lean_words - s0.lean_begin;
+            d.lean[i].stages = P.op_end - P.op_begin;
+        }
+        general = general || (!lean && P.op_begin < P.op_end);
+    }
+    for (const Step &s : p.steps) general = general || s.kind == S_UNBLOCKED;
+    const size_t nc = general ? p.coef.size() : 0;
+    // sections of the device buffer, 256-byte aligned
+    size_t total = 0;
+    auto section = [&](size_t bytes) {
+        const size_t off = total;
+        total += (std::max<size_t>(16, bytes) + 255) & ~size_t(255);
+        return off;
+    };
+    const size_t o_pass = section(p.passes.size() * sizeof(DevPass));
+    const size_t o_ops = section(p.ops.size() * sizeof(DevOp));
+    const size_t o_st = section(stages.size() * sizeof(DevStage));
+    const size_t o_sb = section(p.subs.size() * sizeof(DevSub));
+    const size_t o_tc = section(p.tcs.size() * sizeof(DevTc));
+    const size_t o_im = section(p.tc_images.size());
+    // two spare entries: the register stages read a sub-op's first two coefficients ahead
+    const size_t o_coef = section((nc + 2) * amp_bytes(dt));
+    const size_t o_cdf = section(want_df ? (nc + 2) * 16 : 0);
+    const size_t o_words = section(img.words.size()), o_pool = section(img.pool.size());
     std::vector<unsigned char> h(total, 0);
-    if (!p.passes.empty()) std::memcpy(h.data() + o_pass, p.passes.data(), p.passes.size() * sizeof(DevPass));
-    if (!p.ops.empty()) std::memcpy(h.data() + o_ops, p.ops.data(), p.ops.size() * sizeof(DevOp));
-    if (!p.stages.empty()) std::memcpy(h.data() + o_st, p.stages.data(), p.stages.size() * sizeof(DevStage));
-    if (!p.subs.empty()) std::memcpy(h.data() + o_sb, p.subs.data(), p.subs.size() * sizeof(DevSub));
-    if (!p.tcs.empty()) std::memcpy(h.data() + o_tc, p.tcs.data(), p.tcs.size() * sizeof(DevTc));
-    if (!p.tc_images.empty()) std::memcpy(h.data() + o_im, p.tc_images.data(), p.tc_images.size());
+    auto fill = [&](size_t off, const void *src, size_t bytes) {
+        if (bytes) std::memcpy(h.data() + off, src, bytes);
+    };
+    fill(o_pass, p.passes.data(), p.passes.size() * sizeof(DevPass));
+    fill(o_ops, p.ops.data(), p.ops.size() * sizeof(DevOp));
+    fill(o_st, stages.data(), stages.size() * sizeof(DevStage));
+    fill(o_sb, p.subs.data(), p.subs.size() * sizeof(DevSub));
+    fill(o_tc, p.tcs.data(), p.tcs.size() * sizeof(DevTc));
+    fill(o_im, p.tc_images.data(), p.tc_images.size());
+    fill(o_words, img.words.data(), img.words.size());
+    fill(o_pool, img.pool.data(), img.pool.size());
     if (dt == QS_C64) {
         float *f = reinterpret_cast<float *>(h.data() + o_coef);
-        for (size_t i = 0; i < p.coef.size(); ++i) {
+        for (size_t i = 0; i < nc; ++i) {
             f[2 * i] = (float)p.coef[i].real();
             f[2 * i + 1] = (float)p.coef[i].imag();
         }
     } else {
         double *f = reinterpret_cast<double *>(h.data() + o_coef);
-        for (size_t i = 0; i < p.coef.size(); ++i) {
+        for (size_t i = 0; i < nc; ++i) {
             f[2 * i] = p.coef[i].real();
             f[2 * i + 1] = p.coef[i].imag();
         }
@@ -231,7 +270,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     if (want_df) {
         // each FP64 part x as h = fl32(x), l = fl32(x - h): h + l carries about 48 bits of x
         float *f = reinterpret_cast<float *>(h.data() + o_cdf);
-        for (size_t i = 0; i < p.coef.size(); ++i) {
+        for (size_t i = 0; i < nc; ++i) {
             const double parts[2] = {p.coef[i].real(), p.coef[i].imag()};
             for (int r = 0; r < 2; ++r) {
                 const float hi = (float)parts[r];
@@ -286,6 +325,9 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     d.images = reinterpret_cast<unsigned char *>((char *)base + o_im);
     d.coef = (char *)base + o_coef;
     d.coef_df = want_df ? (char *)base + o_cdf : nullptr;
+    d.words = (char *)base + o_words;
+    d.pool = (char *)base + o_pool;
+    d.h_words = std::move(img.words);
     return QS_OK;
 }
 
@@ -349,8 +391,17 @@ qs_status run_plan(qs_state *s, qs_plan *pl, StepTimer *timer = nullptr, bool tr
             // double-float form: complex128, requested, and a pass of register stages only
             bool df = d.coef_df != nullptr && stp.kind == S_PASS && !hp.has_perm;
             for (int o = hp.op_begin; df && o < hp.op_end; ++o) df = p.ops[o].type == OP_STAGE;
-            const PassArgs pa{d.passes + stp.index, d.ops, d.stages, d.subs, d.coef, rb, d.coef_df, df};
-            rc = launch_pass(c, pa, hp, err, sizeof err);
+            const DevPlanBuf::Lean &L = d.lean[stp.index];
+            if (L.stages > 0) {
+                const LeanPassArgs la{d.h_words.data() + size_t(L.begin) * 16, (const char *)d.words + size_t(L.begin) * 16,
+                                      d.pool, L.words, L.stages, rb, d.coef_df != nullptr};
+                rc = launch_lean_pass(c, la, hp, err, sizeof err);
+            } else {
+                // (the lowered stages of a double-float plan are in that form: not for FP64 passes)
+                const PassArgs pa{d.passes + stp.index, d.ops, d.stages, d.subs, d.coef, rb, d.coef_df, df,
+                                  d.coef_df ? nullptr : d.words, d.pool};
+                rc = launch_pass(c, pa, hp, err, sizeof err);
+            }
             if (stp.kind == S_PASS) s->stats.passes++;
             else s->stats.remaps++;
             s->stats.bytes_moved += pass_bytes;

@@ -16,6 +16,7 @@
 #include <string>
 #include <vector>
 
+#include "lower.h"
 #include "planner.h"
 #include "qs_internal.h"
 
@@ -113,6 +114,7 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     std::vector<DevStage> stages;
     std::vector<DevSub> subs;
     std::vector<cd> coef;
+    LeanImage img;
     B->circs.assign(B->ncirc, BatchCirc{});
     B->items.clear();
     uint64_t amp_off = 0;
@@ -163,7 +165,13 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
             else op.mat += cf_base;
             ops.push_back(op);
         }
-        for (DevStage st : p.stages) {
+        std::vector<DevStage> lowered = p.stages;
+        // complex128 stays on the general engine: with one CTA per SM its descriptor prefetch counts
+        // (59 circuits of 10-15 qubits: 995 us, 1076 us on the in-place engine)
+        if (B->dt == QS_C64) lower_stages(p, B->dt, false, lowered, img);
+        else
+            for (DevStage &st : lowered) st.lean_begin = -1;
+        for (DevStage st : lowered) {
             st.sub_begin += sb_base;
             st.sub_end += sb_base;
             stages.push_back(st);
@@ -196,6 +204,7 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     std::vector<unsigned char> h;
     const size_t o_pass = put(h, passes), o_ops = put(h, ops), o_st = put(h, stages), o_sb = put(h, subs);
     const size_t o_circ = put(h, B->circs), o_item = put(h, B->items);
+    const size_t o_words = put(h, img.words), o_pool = put(h, img.pool);
     const size_t o_coef = (h.size() + 255) & ~size_t(255);
     // two spare entries: the register stages read a sub-op's first two coefficients ahead
     h.resize(o_coef + (coef.size() + 2) * amp_size(B->dt), 0);
@@ -228,6 +237,8 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     a.stages = reinterpret_cast<const DevStage *>(base + o_st);
     a.subs = reinterpret_cast<const DevSub *>(base + o_sb);
     a.coef = base + o_coef;
+    a.words = base + o_words;
+    a.pool = base + o_pool;
     a.done = static_cast<unsigned *>(B->ctl);
     a.head = a.done + B->ndone;
     a.results = reinterpret_cast<double *>(static_cast<char *>(B->ctl) +

@@ -17,7 +17,7 @@
 
 #include <cstdio>
 
-#include "slab_common.cuh"
+#include "lean_stage.cuh"
 
 namespace qs {
 namespace {
@@ -207,8 +207,14 @@ __global__ void __launch_bounds__(NT, 1)
             for (int o = Z.pass.op_begin; o < Z.pass.op_end; ++o) {
                 const DevOp &op = a.ops[o];
                 if ((base & op.ocmask) == op.ocmask) {
-                    if (op.type == OP_STAGE) run_stage<C, RB>(sm, a.stages + op.mat, a.subs, coef, base, tid, NT);
-                    else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
+                    if (op.type == OP_STAGE) {
+                        const DevStage *st = a.stages + op.mat;
+                        if (st->lean_begin >= 0)
+                            run_lean_stage<C, RB>(sm, GlobalWords{static_cast<const ulonglong2 *>(a.words)},
+                                                  uint32_t(st->lean_begin), static_cast<const C *>(a.pool), base, tid);
+                        else
+                            run_stage<C, RB>(sm, st, a.subs, coef, base, tid, NT);
+                    } else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
                 }
                 __syncthreads();
             }

@@ -21,7 +21,7 @@
 
 #include <cstdio>
 
-#include "slab_common.cuh"
+#include "lean_stage.cuh"
 
 namespace qs {
 
@@ -47,7 +47,8 @@ __global__ void __launch_bounds__(NT, 1)
     slab_pass_kernel(typename Cx<R>::T *__restrict__ state, const DevPass *__restrict__ d_pass,
                      const DevOp *__restrict__ ops, const DevStage *__restrict__ stages,
                      const DevSub *__restrict__ subs, const typename Cx<R>::T *__restrict__ coef,
-                     const dfc *__restrict__ coef_df, uint64_t nslabs)
+                     const dfc *__restrict__ coef_df, const ulonglong2 *__restrict__ words,
+                     const typename Cx<R>::T *__restrict__ pool, uint64_t nslabs)
 {
     using C = typename Cx<R>::T;
     static_assert(!DF || sizeof(C) == sizeof(dfc), "double-float slabs replace complex128 slabs");
@@ -156,8 +157,12 @@ __global__ void __launch_bounds__(NT, 1)
             for (int o = op_begin; o < op_end; ++o) {
                 const DevOp &op = ops[o];
                 if ((base & op.ocmask) == op.ocmask) {
-                    if (op.type == OP_STAGE) run_stage<C, RB>(sm, stages + op.mat, subs, coef, base, tid, NT);
-                    else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
+                    if (op.type == OP_STAGE) {
+                        const DevStage *st = stages + op.mat;
+                        if (words != nullptr && st->lean_begin >= 0)
+                            run_lean_stage<C, RB>(sm, GlobalWords{words}, uint32_t(st->lean_begin), pool, base, tid);
+                        else run_stage<C, RB>(sm, st, subs, coef, base, tid, NT);
+                    } else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
                 }
                 __syncthreads();
             }
@@ -209,7 +214,8 @@ int launch_pass_t(const LaunchCtx &c, const PassArgs &a, const DevPass &h, char 
     if (grid > nslabs) grid = nslabs;
     slab_pass_kernel<R, RB, NT, DF><<<(unsigned)grid, NT, smem, (cudaStream_t)c.stream>>>(
         reinterpret_cast<C *>(c.amp), a.pass, a.ops, a.stages, a.subs,
-        reinterpret_cast<const C *>(a.coef), reinterpret_cast<const dfc *>(a.coef_df), nslabs);
+        reinterpret_cast<const C *>(a.coef), reinterpret_cast<const dfc *>(a.coef_df),
+        static_cast<const ulonglong2 *>(a.words), static_cast<const C *>(a.pool), nslabs);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         snprintf(err, errlen, "slab pass launch failed: %s", cudaGetErrorString(e));

@@ -107,7 +107,35 @@ struct DevStage {
     uint8_t rest[16];   // non-register slab-local bits; group index bit j -> rest[j]
     uint16_t off[32];   // slab-local offset of register index e
     int32_t sub_begin, sub_end;
+    // the stage for the in-place engine (lower.cpp, lean_stage.cuh): its first 16-byte word, or
+    // lean_begin < 0 where the stage holds a sub-op that only the general engine runs
+    int32_t lean_begin, lean_words;
 };
+
+// Words of a lowered stage.  Head: {u8 register bit positions[RB] (8 bytes), u32 nrest | flip << 8,
+// u32 number of words that follow}; flip: register bits whose two values the stage exchanges when it
+// stores.  Then records, each starting with a word {u8 op, a, b, ndl, u32 arg, ...}; "conditions" is a
+// word {u32 slab-local bits, -, u64 outside bits} that must all be 1.
+enum LeanOp : uint8_t {
+    L_ROT0 = 0,   // L_ROT0 + j: (y, x) of register bit j, complex64 in the word's upper half, else in
+                  // a word of its own: v1 += y v0; v0 += x v1.  FP64: v0 + x v1, y v0 + v1 (old
+                  // values)
+    L_ROT1, L_ROT2, L_ROT3, L_ROT4,
+    L_ROTM0,      // FP64: v0 + x v1, y v0 - v1
+    L_ROTM1, L_ROTM2, L_ROTM3,
+    L_ROTA,       // complex64: (y, x) of every register bit, from the upper half on, two per word
+    L_CONST,      // u32 at byte 8 = pattern that holds the factors other than 1; all factors follow
+    L_TABLE,      // arg = first word in the pool; byte 8 as L_CONST; ndl condition bits, the first b of
+                  // them inside the slab; a word of condition codes u8[12] (as DevSub::dl)
+    L_SCALE,      // real factors follow
+    L_SIGN,       // arg = elements whose sign changes; conditions
+    L_PHASE,      // arg = elements; byte 8 = pattern that holds them; conditions; the factor
+    L_CX,         // X on register bit a, register control b (0xff: none); conditions
+};
+// Tables are stored [conditions outside the slab][e >> p][conditions inside it][e & (2^p - 1)]:
+// lanes of a warp that differ in a condition bit read neighbouring 16-byte words, and one slab
+// reads one contiguous part.  A complex64 word holds two entries: both real, both imaginary parts.
+constexpr int lean_pair_log(qs_dtype dt) { return dt == QS_C64 ? 1 : 0; }
 
 int num_sms();
 
@@ -150,7 +178,17 @@ struct PassArgs {
     int stage_bits;           // register-stage width the plan was built for
     const void *coef_df;      // device, whole plan, double-float quadruples (or NULL)
     bool df;                  // complex128 pass of register stages only, in double-float form
+    const void *words;        // device, whole plan: lowered stages (NULL: use the general engine) ...
+    const void *pool;         // ... and their conditional tables
 };
+// A pass of lowered register stages only, without a store permutation (k_lean.cu): h_words, its
+// words on the host (nwords of them, nstages stages); d_words, the same on the device.
+struct LeanPassArgs {
+    const void *h_words, *d_words, *pool;
+    int nwords, nstages, stage_bits;
+    bool df;
+};
+int launch_lean_pass(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h_pass, char *err, size_t errlen);
 int launch_pass(const LaunchCtx &c, const PassArgs &a, const DevPass &h_pass, char *err,
                 size_t errlen);
 // Device status word written by bounded waits that ran out (0 = fine).  Reading clears it.
@@ -188,6 +226,8 @@ struct BatchArgs {
     const DevStage *stages;
     const DevSub *subs;
     const void *coef;
+    const void *words;  // lowered stages and their conditional tables
+    const void *pool;
     const BatchTerm *terms;
     unsigned *done;     // per circuit per pass: slabs stored (zeroed before each run)
     unsigned *head;     // work-queue head (zeroed before each run)
