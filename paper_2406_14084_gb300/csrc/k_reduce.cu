@@ -19,6 +19,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "qs_internal.h"
@@ -337,123 +338,156 @@ __global__ void __launch_bounds__(kRedThreads) expect_wht_kernel(const typename 
     }
 }
 
-// Marginal probabilities: hist[m] += |a_x|^2 with m gathered from the bits pos[0..nq).
+// Marginal probabilities: hist[m] = sum of |a_x|^2 over the x whose bits pos[0..nq) read m.
+//
+// The index bits fall into three parts: the low ones, which the 32 lanes (and the two amplitudes of a
+// 16-byte complex64 load) cover; the selected bits above them, fixed for a warp; and the other bits
+// above, which the warp runs over.  Each lane so adds into one or two sums that belong to one bin
+// whatever nq is; at the end lanes of the same bin are added with shuffles, the eight warps of a CTA in
+// shared memory where they share their bins, and the rest with one FP64 atomic per CTA or warp and bin
+// (none where a bin belongs to one warp).  Bound by HBM (complex64) or the FP64 pipe (complex128, two
+// FMAs per amplitude).  The kernels before added each amplitude into a shared-memory histogram with an
+// FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.22) or kept every bin in registers with one
+// select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.39).
+struct ProbsPlan {
+    uint64_t hs, hn;      // selected / other bits above the low ones
+    int ns, nn, logc;     // their counts; log2 of the warps that share one setting of hs
+    int low, nq;          // number of low bits
+    uint8_t pos[32];
+};
+
+// the i-th (bit-wise) subset of mask
+__device__ __forceinline__ uint64_t deposit(uint64_t i, uint64_t mask)
+{
+    uint64_t r = 0;
+    for (; i != 0; i >>= 1, mask &= mask - 1)
+        if (i & 1) r |= mask & (~mask + 1);
+    return r;
+}
+
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>::T *__restrict__ a,
-                                                            uint64_t N, int nq, uint4 pos_packed0,
-                                                            uint4 pos_packed1,
-                                                            double *__restrict__ hist)
+                                                            const __grid_constant__ ProbsPlan p, double *__restrict__ hist)
 {
-    extern __shared__ double sh[];
-    const int M = 1 << nq;
-    const bool use_smem = nq <= 11;
-    if (use_smem)
-        for (int m = threadIdx.x; m < M; m += blockDim.x) sh[m] = 0.0;
-    __syncthreads();
-    uint8_t pos[32];
-    const uint32_t w[8] = {pos_packed0.x, pos_packed0.y, pos_packed0.z, pos_packed0.w,
-                           pos_packed1.x, pos_packed1.y, pos_packed1.z, pos_packed1.w};
+    using T = typename Cx<R>::T;
+    constexpr int VL = sizeof(T) == 8 ? 1 : 0;  // low bit inside a 16-byte load
+    constexpr int U = 8;                        // loads in flight per lane
+    __shared__ double sh[kRedThreads / 32][32][1 << VL];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t units = 1ull << (p.ns + p.logc);
+    const uint64_t mine = uint64_t(lane) << VL;
+    const bool live = (mine >> p.low) == 0;  // states smaller than one load per lane
+    const int nrun = p.nn - p.logc;          // bits of hn that one warp runs over: the low nrun ones
+    const uint64_t chunk = nrun >= 64 ? 0 : deposit(~0ull << nrun & ((1ull << p.nn) - 1), p.hn);  // the others
+    const uint64_t run = p.hn & ~chunk;
+    uint64_t off[U], rest = run;  // off: the loads in flight
+    int nu = 0;  // the lowest bits of run, up to three, index the loads in flight
+    for (; nu < 3 && rest != 0; ++nu) rest &= rest - 1;
+    const uint64_t inner = run & ~rest;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) pos[j] = (w[j >> 2] >> (8 * (j & 3))) & 0xff;
-    const uint64_t per = (N + gridDim.x - 1) / gridDim.x;
-    const uint64_t lo = per * blockIdx.x;
-    const uint64_t hi = lo + per < N ? lo + per : N;
-    for (uint64_t x = lo + threadIdx.x; x < hi; x += blockDim.x) {
-        const auto v = a[x];
-        const double p = (double)v.x * (double)v.x + (double)v.y * (double)v.y;
-        uint32_t m = 0;
+    for (int u = 0; u < U; ++u) off[u] = deposit(uint64_t(u) & ((1u << nu) - 1), inner);
+    const uint64_t iters = 1ull << (nrun - nu);
+    const bool joint = p.logc >= 3;  // the CTA's warps share hs
+    for (uint64_t u0 = uint64_t(blockIdx.x) * (kRedThreads / 32); u0 < units;
+         u0 += uint64_t(gridDim.x) * (kRedThreads / 32)) {
+        const uint64_t unit = u0 + warp;
+        const bool has = unit < units;
+        const uint64_t fixed = deposit(unit >> p.logc, p.hs) | deposit(unit & ((1ull << p.logc) - 1), chunk) | mine;
+        double acc[1 << VL] = {};
+        R f[1 << VL] = {};
+        auto add = [&](const auto &v) {  // one load's amplitudes
+            if constexpr (VL == 1) {
+                f[0] = fmaf(v.x, v.x, f[0]);
+                f[0] = fmaf(v.y, v.y, f[0]);
+                f[VL] = fmaf(v.z, v.z, f[VL]);
+                f[VL] = fmaf(v.w, v.w, f[VL]);
+            } else {
+                acc[0] = fma(v.x, v.x, acc[0]);
+                acc[0] = fma(v.y, v.y, acc[0]);
+            }
+        };
+        using V = std::conditional_t<VL == 1, float4, double2>;
+        if (has && live) {
+            if (nu == 3) {
+                uint64_t x = 0;
+                for (uint64_t it = 0; it < iters; ++it) {
+                    V v[U];
 #pragma unroll
-        for (int j = 0; j < 32; ++j)  // unrolled so that pos[] stays in registers
-            if (j < nq) m |= uint32_t((x >> pos[j]) & 1) << j;
-        if (use_smem) atomicAdd(&sh[m], p);
-        else atomicAdd(&hist[m], p);
-    }
-    if (use_smem) {
-        __syncthreads();
-        for (int m = threadIdx.x; m < M; m += blockDim.x)
-            if (sh[m] != 0.0) atomicAdd(&hist[m], sh[m]);
+                    for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const V *>(a + (fixed | x | off[u])));
+#pragma unroll
+                    for (int u = 0; u < U; ++u) add(v[u]);
+                    if (VL == 1 && (it & 3) == 3) {  // FP32 partial sums of at most 32 amplitudes
+                        acc[0] += (double)f[0];
+                        acc[VL] += (double)f[VL];
+                        f[0] = f[VL] = R(0);
+                    }
+                    x = ((x | ~rest) + 1) & rest;  // the next subset of rest
+                }
+            } else {  // fewer than eight loads in all
+                for (uint32_t u = 0; u < (1u << nu); ++u)
+                    add(__ldcs(reinterpret_cast<const V *>(a + (fixed | deposit(u, inner)))));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < (1 << VL); ++k) acc[k] += (double)f[k];
+        // lanes (and halves) of one bin; selected low bits keep them apart
+        uint32_t keep = 0;
+        for (int j = 0; j < p.nq; ++j)
+            if (p.pos[j] < p.low) keep |= 1u << p.pos[j];
+        if (VL == 1 && !(keep & 1u)) {
+            acc[0] += acc[VL];
+            acc[VL] = acc[0];
+        }
+        bool writer = true;
+        for (int l = 0; l < 5; ++l) {
+            if (keep >> (l + VL) & 1u) continue;
+#pragma unroll
+            for (int k = 0; k < (1 << VL); ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 1 << l);
+            writer = writer && !(lane >> l & 1);
+        }
+        if (joint) {
+#pragma unroll
+            for (int k = 0; k < (1 << VL); ++k) sh[warp][lane][k] = acc[k];
+            __syncthreads();
+            if (warp == 0) {
+#pragma unroll
+                for (int k = 0; k < (1 << VL); ++k)
+                    for (int w = 1; w < kRedThreads / 32; ++w) acc[k] += sh[w][lane][k];
+            }
+            __syncthreads();
+            writer = writer && warp == 0;
+        }
+        if (writer && has && live) {
+            const uint64_t x = deposit(unit >> p.logc, p.hs) | mine;
+            const int halves = VL == 1 && (keep & 1u) ? 2 : 1;
+            for (int k = 0; k < halves; ++k) {
+                uint32_t m = 0;
+                for (int j = 0; j < p.nq; ++j) m |= uint32_t(((x | uint64_t(k)) >> p.pos[j]) & 1) << j;
+                if (p.logc == 0) hist[m] = acc[k];
+                else atomicAdd(&hist[m], acc[k]);
+            }
+        }
     }
 }
 
-// Marginals over at most Q qubits (2^Q bins): each thread keeps its bins in registers
-// (branch-free select-and-add per bin), then the bins are reduced with warp shuffles and added
-// to the global histogram with one FP64 atomic per warp and bin.
-template <typename R, int Q>
-__global__ void __launch_bounds__(kRedThreads) probs_small_kernel(const typename Cx<R>::T *__restrict__ a,
-                                                                  uint64_t N, int nq, uint4 pos_packed0,
-                                                                  double *__restrict__ hist)
+ProbsPlan probs_plan(int n, qs_dtype dt, const int *pos, int nq)
 {
-    constexpr int M = 1 << Q;
-    uint32_t pos[Q];
-    const uint32_t w[4] = {pos_packed0.x, pos_packed0.y, pos_packed0.z, pos_packed0.w};
-#pragma unroll
-    for (int j = 0; j < Q; ++j) pos[j] = (w[j >> 2] >> (8 * (j & 3))) & 0xff;
-    // complex64: FP32 partial sums of at most 32 amplitudes per bin, then FP64 (the FP64 pipe
-    // is 1/64 of the FP32 rate on this part); with at most 8 bins, 32 of those partials are first
-    // summed in FP32 (converting every one kept the FP64 pipe 40 % busy on 3-qubit marginals;
-    // 32 bins would not fit the second level in registers); complex128: FP64 throughout
-    constexpr bool kTwoLevel = M <= 8;
-    double acc[M];
-    R part[M], part2[M];
-#pragma unroll
-    for (int b = 0; b < M; ++b) {
-        acc[b] = 0.0;
-        part[b] = part2[b] = R(0);
+    ProbsPlan p{};
+    p.low = std::min(n, dt == QS_C64 ? 6 : 5);
+    p.nq = nq;
+    uint64_t sel = 0;
+    for (int j = 0; j < nq; ++j) {
+        p.pos[j] = uint8_t(pos[j]);
+        sel |= 1ull << pos[j];
     }
-    int cnt = 0, cnt2 = 0;
-    const uint64_t per = (N + gridDim.x - 1) / gridDim.x;
-    const uint64_t lo = per * blockIdx.x;
-    const uint64_t hi = lo + per < N ? lo + per : N;
-    constexpr int U = 4;  // independent loads in flight per thread
-    using T = typename Cx<R>::T;
-    for (uint64_t x0 = lo + threadIdx.x; x0 < hi; x0 += uint64_t(U) * blockDim.x) {
-        T v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint64_t x = x0 + uint64_t(u) * blockDim.x;
-            v[u] = x < hi ? a[x] : T{};  // past the range: weight 0
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint64_t x = x0 + uint64_t(u) * blockDim.x;
-            const R p = (R)v[u].x * (R)v[u].x + (R)v[u].y * (R)v[u].y;
-            uint32_t m = 0;
-#pragma unroll
-            for (int j = 0; j < Q; ++j)
-                if (j < nq) m |= uint32_t((x >> pos[j]) & 1) << j;
-            if (sizeof(R) == 8) {
-#pragma unroll
-                for (int b = 0; b < M; ++b) acc[b] += (m == uint32_t(b)) ? (double)p : 0.0;
-            } else {
-#pragma unroll
-                for (int b = 0; b < M; ++b) part[b] += (m == uint32_t(b)) ? p : R(0);
-            }
-        }
-        if (sizeof(R) == 4 && (cnt += U) >= 32) {
-#pragma unroll
-            for (int b = 0; b < M; ++b) {
-                part2[b] += part[b];
-                part[b] = R(0);
-            }
-            cnt = 0;
-            if (!kTwoLevel || ++cnt2 == 32) {
-#pragma unroll
-                for (int b = 0; b < M; ++b) {
-                    acc[b] += (double)part2[b];
-                    part2[b] = R(0);
-                }
-                cnt2 = 0;
-            }
-        }
-    }
-#pragma unroll
-    for (int b = 0; b < M; ++b) acc[b] += (double)part[b] + (double)part2[b];
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int b = 0; b < M; ++b) {
-        const double t = warp_sum(acc[b]);
-        if (lane == 0 && b < (1 << nq) && t != 0.0) atomicAdd(&hist[b], t);
-    }
+    const uint64_t above = ((1ull << n) - 1) & ~((1ull << p.low) - 1);
+    p.hs = sel & above;
+    p.hn = above & ~sel;
+    p.ns = __builtin_popcountll(p.hs);
+    p.nn = __builtin_popcountll(p.hn);
+    // 2^13 warps fill the GPU (6.7 CTAs of eight per SM); below eight loads per warp fewer share a bin
+    p.logc = std::max(0, std::min(13 - p.ns, p.nn - 3));
+    return p;
 }
 
 int g_sms = 0;
@@ -509,41 +543,34 @@ int launch_norm2(const LaunchCtx &c, double *d_scratch, double *h_out, char *err
     return QS_OK;
 }
 
+namespace {
+
+int enqueue_probs(const LaunchCtx &c, const int *phys_q, int nq, double *hist, char *err, size_t errlen)
+{
+    cudaStream_t st = (cudaStream_t)c.stream;
+    const ProbsPlan p = probs_plan(c.n, c.dt, phys_q, nq);
+    if (p.logc > 0 && cudaMemsetAsync(hist, 0, (size_t(1) << nq) * sizeof(double), st) != cudaSuccess)
+        return cuda_fail("probs memset", err, errlen);
+    reduce_blocks(1);  // reads the SM count once
+    const uint64_t need = ((1ull << (p.ns + p.logc)) + kRedThreads / 32 - 1) / (kRedThreads / 32);
+    const int blocks = int(std::min<uint64_t>(need, uint64_t(g_sms) * 8));
+    if (c.dt == QS_C64) probs_kernel<float><<<blocks, kRedThreads, 0, st>>>((const float2 *)c.amp, p, hist);
+    else probs_kernel<double><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, p, hist);
+    return cuda_fail("probs launch", err, errlen);
+}
+
+}  // namespace
+
 int launch_probs(const LaunchCtx &c, const int *phys_q, int nq, double *d_scratch,
                  size_t scratch_bytes, double *h_out, char *err, size_t errlen)
 {
-    const uint64_t N = 1ull << c.n;
     const size_t M = size_t(1) << nq;
     if (M * sizeof(double) > scratch_bytes) {
         snprintf(err, errlen, "probs: scratch too small");
         return QS_EINVAL;
     }
     cudaStream_t st = (cudaStream_t)c.stream;
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < nq; ++j) w[j >> 2] |= uint32_t(phys_q[j] & 0xff) << (8 * (j & 3));
-    uint4 p0 = make_uint4(w[0], w[1], w[2], w[3]), p1 = make_uint4(w[4], w[5], w[6], w[7]);
-    if (cudaMemsetAsync(d_scratch, 0, M * sizeof(double), st) != cudaSuccess)
-        return cuda_fail("probs memset", err, errlen);
-    const int blocks = reduce_blocks(N);
-    const size_t smem = nq <= 11 ? M * sizeof(double) : 0;
-    if (nq <= 3) {
-        if (c.dt == QS_C64)
-            probs_small_kernel<float, 3><<<blocks, kRedThreads, 0, st>>>((const float2 *)c.amp, N, nq, p0, d_scratch);
-        else
-            probs_small_kernel<double, 3><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, N, nq, p0, d_scratch);
-    } else if (nq <= 5) {
-        if (c.dt == QS_C64)
-            probs_small_kernel<float, 5><<<blocks, kRedThreads, 0, st>>>((const float2 *)c.amp, N, nq, p0, d_scratch);
-        else
-            probs_small_kernel<double, 5><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, N, nq, p0, d_scratch);
-    } else if (c.dt == QS_C64) {
-        probs_kernel<float><<<blocks, kRedThreads, smem, st>>>((const float2 *)c.amp, N, nq, p0, p1,
-                                                               d_scratch);
-    } else {
-        probs_kernel<double><<<blocks, kRedThreads, smem, st>>>((const double2 *)c.amp, N, nq, p0,
-                                                                p1, d_scratch);
-    }
-    int rc = cuda_fail("probs launch", err, errlen);
+    int rc = enqueue_probs(c, phys_q, nq, d_scratch, err, errlen);
     if (rc) return rc;
     if (cudaMemcpyAsync(h_out, d_scratch, M * sizeof(double), cudaMemcpyDeviceToHost, st) !=
             cudaSuccess ||
@@ -725,24 +752,9 @@ int launch_probs_static(const LaunchCtx &c, const int *phys_q, int nq, double *h
     double *hist = nullptr;
     int rc = static_probs_scratch(&hist, err, errlen);
     if (rc) return rc;
-    const uint64_t N = 1ull << c.n;
     const size_t M = size_t(1) << nq;
     cudaStream_t st = (cudaStream_t)c.stream;
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < nq; ++j) w[j >> 2] |= uint32_t(phys_q[j] & 0xff) << (8 * (j & 3));
-    uint4 p0 = make_uint4(w[0], w[1], w[2], w[3]), p1 = make_uint4(w[4], w[5], w[6], w[7]);
-    // the array keeps the previous call's histogram: clear the bins this call accumulates into
-    if (cudaMemsetAsync(hist, 0, M * sizeof(double), st) != cudaSuccess)
-        return cuda_fail("probs_noalloc memset", err, errlen);
-    const int blocks = reduce_blocks(N);
-    const size_t smem = nq <= 11 ? M * sizeof(double) : 0;
-    if (c.dt == QS_C64)
-        probs_kernel<float><<<blocks, kRedThreads, smem, st>>>((const float2 *)c.amp, N, nq, p0, p1,
-                                                               hist);
-    else
-        probs_kernel<double><<<blocks, kRedThreads, smem, st>>>((const double2 *)c.amp, N, nq, p0,
-                                                                p1, hist);
-    rc = cuda_fail("probs_noalloc launch", err, errlen);
+    rc = enqueue_probs(c, phys_q, nq, hist, err, errlen);
     if (rc) return rc;
     if (cudaMemcpyAsync(h_out, hist, M * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
