@@ -20,6 +20,7 @@
 #include <cstring>
 #include <mutex>
 #include <type_traits>
+#include <unordered_map>
 #include <vector>
 
 #include "qs_internal.h"
@@ -93,9 +94,9 @@ __global__ void __launch_bounds__(kRedThreads) norm2_kernel(const typename Cx<R>
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-// Sum `count` pairs (re, im) laid out as part[i], part[stride + i]; writes out[0], out[1].
+// Sum `count` pairs (re, im) laid out as part[i], part[stride + i]; writes out[0], out[1], or adds to them.
 __global__ void __launch_bounds__(kRedThreads) finish_kernel(const double *__restrict__ part, int count,
-                                                             int stride, double *__restrict__ out)
+                                                             int stride, double *__restrict__ out, bool add)
 {
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < count; i += blockDim.x) {
@@ -104,8 +105,8 @@ __global__ void __launch_bounds__(kRedThreads) finish_kernel(const double *__res
     }
     block_sum2(a, b);
     if (threadIdx.x == 0) {
-        out[0] = a;
-        out[1] = b;
+        out[0] = add ? out[0] + a : a;
+        out[1] = add ? out[1] + b : b;
     }
 }
 
@@ -518,8 +519,9 @@ int cuda_fail(const char *what, char *err, size_t errlen)
 
 size_t reduce_scratch_bytes()
 {
-    // partials (2 x blocks) + 2 results + one term group + its Walsh-Hadamard term table
-    return sizeof(double) * (2 * kRedBlocksMax + 8) + sizeof(TermGroup) + 256 + sizeof(WhtTerms) + 256;
+    // partials (2 x blocks) + 2 results + one term group + its Walsh-Hadamard term table + one tile's groups
+    return sizeof(double) * (2 * kRedBlocksMax + 8) + sizeof(TermGroup) + 256 + sizeof(WhtTerms) + 256 +
+           pauli_tile_bytes() + 256;
 }
 
 int launch_norm2(const LaunchCtx &c, double *d_scratch, double *h_out, char *err, size_t errlen)
@@ -532,7 +534,7 @@ int launch_norm2(const LaunchCtx &c, double *d_scratch, double *h_out, char *err
         norm2_kernel<float><<<blocks, kRedThreads, 0, st>>>((const float2 *)c.amp, N, part);
     else
         norm2_kernel<double><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, N, part);
-    finish_kernel<<<1, kRedThreads, 0, st>>>(part, blocks, 0, res);
+    finish_kernel<<<1, kRedThreads, 0, st>>>(part, blocks, 0, res, false);
     int rc = cuda_fail("norm2 launch", err, errlen);
     if (rc) return rc;
     double r[2];
@@ -625,27 +627,63 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
     double *part = d_scratch, *res = d_scratch + 2 * kRedBlocksMax;
     TermGroup *dgrp = reinterpret_cast<TermGroup *>(d_scratch + 2 * kRedBlocksMax + 8);
     const int blocks = reduce_blocks(N);
-    std::vector<TermGroup> hgv(1);  // host staging; each copy completes before reuse
+    auto aligned = [](void *p) { return (reinterpret_cast<uintptr_t>(p) + 255) & ~uintptr_t(255); };
+    WhtTerms *dpt = reinterpret_cast<WhtTerms *>(aligned(dgrp + 1));
+    void *dtile = reinterpret_cast<void *>(aligned(dpt + 1));
+    // Terms by X mask, in order of first appearance, at most kMaxTermsPerGroup each.  (Host staging: a
+    // copy from pageable memory has left it when the call returns.)
+    std::vector<PauliXGroup> groups;
+    {
+        std::unordered_map<uint64_t, int> open;  // X mask -> the group that still takes terms
+        for (size_t i = 0; i < nterms; ++i) {
+            auto it = open.find(xm[i]);
+            if (it == open.end() || groups[it->second].zm.size() == size_t(kMaxTermsPerGroup)) {
+                open[xm[i]] = int(groups.size());
+                groups.push_back(PauliXGroup{xm[i], {}, {}});
+                it = open.find(xm[i]);
+            }
+            groups[it->second].zm.push_back(zm[i]);
+            groups[it->second].c.push_back(coeff[i]);
+        }
+    }
+    if (cudaMemsetAsync(res, 0, 2 * sizeof(double), st) != cudaSuccess) return cuda_fail("expect memset", err, errlen);
+    // X masks with few terms share reads of the state (k_pauli.cu).  A term costs a tile pass about 2
+    // operations per pair of amplitudes, so up to 8 terms per mask are well below a pass of their own.
+    std::vector<int> tiles;
+    std::vector<char> done(groups.size(), 0);
+    for (size_t g = 0; g < groups.size(); ++g)
+        if (groups[g].xm != 0 && groups[g].zm.size() <= 8) tiles.push_back(int(g));
+    std::vector<char> htile(pauli_tile_bytes());
+    while (!tiles.empty()) {
+        const std::vector<int> before = tiles;
+        const int b = pauli_tile_plan(c, groups, tiles, htile.data());
+        if (b == 0) {
+            tiles.erase(tiles.begin());  // more X bits than a tile holds: a pass of its own below
+            continue;
+        }
+        for (int g : before) done[g] = 1;
+        for (int g : tiles) done[g] = 0;
+        if (cudaMemcpyAsync(dtile, htile.data(), htile.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+            return cuda_fail("expect upload", err, errlen);
+        const int nblk = launch_pauli_tile(c, dtile, b, part, kRedBlocksMax);
+        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
+        int rc = cuda_fail("expect launch", err, errlen);
+        if (rc) return rc;
+    }
+    std::vector<TermGroup> hgv(1);
     TermGroup &hg = hgv[0];
     std::vector<WhtTerms> hw(1);
-    WhtTerms *dpt = reinterpret_cast<WhtTerms *>(
-        (reinterpret_cast<uintptr_t>(dgrp) + sizeof(TermGroup) + 255) & ~uintptr_t(255));
-    double tot_r = 0.0, tot_i = 0.0;
-    std::vector<char> done(nterms, 0);
-    for (size_t i = 0; i < nterms; ++i) {
-        if (done[i]) continue;
-        // gather all not-yet-done terms with this X mask (up to the group capacity)
-        hg.xm = xm[i];
-        hg.nterms = 0;
-        for (size_t j = i; j < nterms && hg.nterms < kMaxTermsPerGroup; ++j) {
-            if (done[j] || xm[j] != xm[i]) continue;
-            done[j] = 1;
-            const int ny = __builtin_popcountll(xm[j] & zm[j]) & 3;
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+        if (done[gi]) continue;
+        const PauliXGroup &G = groups[gi];
+        hg.xm = G.xm;
+        hg.nterms = int(G.zm.size());
+        for (int j = 0; j < hg.nterms; ++j) {
+            const int ny = __builtin_popcountll(G.xm & G.zm[j]) & 3;
             static const double pr[4] = {1, 0, -1, 0}, pi[4] = {0, 1, 0, -1};
-            hg.zm[hg.nterms] = zm[j];
-            hg.cre[hg.nterms] = coeff[j] * pr[ny];
-            hg.cim[hg.nterms] = coeff[j] * pi[ny];
-            hg.nterms++;
+            hg.zm[j] = G.zm[j];
+            hg.cre[j] = G.c[j] * pr[ny];
+            hg.cim[j] = G.c[j] * pi[ny];
         }
         int nblk = blocks;
         if (hg.nterms >= 4 && c.n >= 16) {
@@ -684,18 +722,13 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
                 expect_kernel<double><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, N, dgrp,
                                                                       part);
         }
-        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res);
+        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
         int rc = cuda_fail("expect launch", err, errlen);
         if (rc) return rc;
-        double r[2];
-        if (cudaMemcpyAsync(r, res, sizeof(r), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return cuda_fail("expect readback", err, errlen);
-        tot_r += r[0];
-        tot_i += r[1];
     }
-    h_out[0] = tot_r;
-    h_out[1] = tot_i;
+    if (cudaMemcpyAsync(h_out, res, 2 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return cuda_fail("expect readback", err, errlen);
     return QS_OK;
 }
 

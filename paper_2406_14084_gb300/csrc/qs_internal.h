@@ -13,6 +13,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <vector>
 
 #include "qs.h"
 
@@ -249,6 +250,16 @@ int launch_probs(const LaunchCtx &c, const int *phys_q, int nq, double *d_scratc
 int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm,
                   const double *coeff, size_t nterms, double *d_scratch, size_t scratch_bytes,
                   double *h_out, char *err, size_t errlen);
+// Pauli strings with one X mask (physical masks); groups with few terms are evaluated several X masks
+// per read of the state (k_pauli.cu).
+struct PauliXGroup {
+    uint64_t xm;
+    std::vector<uint64_t> zm;
+    std::vector<double> c;
+};
+size_t pauli_tile_bytes();
+int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, std::vector<int> &todo, void *h_tile);
+int launch_pauli_tile(const LaunchCtx &c, const void *d_tile, int b, double *part, int max_blocks);  // blocks used
 int launch_set_basis(const LaunchCtx &c, uint64_t x, char *err, size_t errlen);
 
 // Measurement sampling (k_sample.cu): d_out[k] = outcome of uniform d_u[k]; the scratch must

@@ -1,8 +1,10 @@
 """Readout kernels at the edges of their splits, against the FP64 oracle on the same amplitudes.
 
 Marginals: states smaller than one load per lane, selections of low bits only, high bits only and both,
-every bin count from the norm to all qubits, one and several loads per warp.  Tolerances as in
-test_gpu_parity.py: 1e-12 / 1e-6 for probabilities."""
+every bin count from the norm to all qubits, one and several loads per warp.  Pauli sums: few-term X
+masks inside one tile, spread over several, and wider than any tile, with odd and even numbers of Y,
+next to groups that go through the other kernels.  Tolerances as in test_gpu_parity.py: 1e-12 / 1e-6
+for probabilities, 1e-9 n / 1e-4 n for expectations."""
 import numpy as np
 import pytest
 
@@ -46,3 +48,26 @@ def test_marginals_of_all_qubits(dtype):
         qs.qs_copy_from_host(s.h, v)
         order = W.SplitMix64(2).distinct(n, n)
         assert np.max(np.abs(s.probs(order) - oracle.probs(ref, n, order))) <= PTOL[dtype]
+
+
+@pytest.mark.parametrize("dtype", [qs.QS_C64, qs.QS_C128])
+@pytest.mark.parametrize("n", [1, 2, 3, 8, 12, 13, 15, 18])
+def test_few_term_x_masks(n, dtype):
+    v, ref = state(n, dtype, 50 + n)
+    sm = W.SplitMix64(n)
+    full = (1 << n) - 1
+    terms = [(1.0, full, 0), (0.5, full, full), (-0.7, full, 1), (0.3, 0, full)]
+    for i in range(n - 1):
+        pair = 3 << i
+        terms += [(0.4 + 0.1 * i, pair, 0), (0.3, pair, pair), (0.2, 0, pair), (-0.6, pair, 1 << i)]
+    for i in range(90):  # scattered masks, many Z bits, some masks more than once
+        terms.append((2.0 * sm.uniform() - 1.0, sm.next_u64() & sm.next_u64() & full, sm.next_u64() & full))
+    for i in range(20):  # one mask with more terms than a tile takes
+        terms.append((0.05 * i, 1 << (n - 1), sm.next_u64() & full))
+    tol = (1e-9 if dtype == qs.QS_C128 else 1e-4) * n
+    with qs.State(n, dtype) as s:
+        qs.qs_copy_from_host(s.h, v)
+        for part in (terms, terms[:1], terms[4:12], [t for t in terms if t[1]]):
+            want = oracle.expect_pauli(ref, n, part)
+            got = s.expect(part)
+            assert abs(got.real - want.real) <= tol and abs(got.imag - want.imag) <= tol
