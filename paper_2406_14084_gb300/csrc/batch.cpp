@@ -115,6 +115,9 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     std::vector<DevSub> subs;
     std::vector<cd> coef;
     LeanImage img;
+    std::vector<BatchProg> progs;
+    uint32_t max_words = 16;
+    bool lean = B->dt == QS_C64;  // so far every pass consists of lowered stages
     B->circs.assign(B->ncirc, BatchCirc{});
     B->items.clear();
     uint64_t amp_off = 0;
@@ -166,11 +169,21 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
             ops.push_back(op);
         }
         std::vector<DevStage> lowered = p.stages;
-        // complex128 stays on the general engine: with one CTA per SM its descriptor prefetch counts
-        // (59 circuits of 10-15 qubits: 995 us, 1076 us on the in-place engine)
-        if (B->dt == QS_C64) lower_stages(p, B->dt, false, lowered, img);
-        else
-            for (DevStage &st : lowered) st.lean_begin = -1;
+        // complex128 runs on the general engine (k_batch.cu)
+        if (lean) lower_stages(p, B->dt, false, lowered, img);
+        for (const Step &s : p.steps) {
+            const DevPass &P = p.passes[s.index];
+            BatchProg g{0, 0, 0, 0};
+            for (int o = P.op_begin; lean && o < P.op_end; ++o)
+                lean = p.ops[o].type == OP_STAGE && lowered[p.ops[o].mat].lean_begin >= 0;
+            if (lean && P.op_begin < P.op_end) {  // the stages of a pass, and so their words, are consecutive
+                const DevStage &s0 = lowered[p.ops[P.op_begin].mat], &s1 = lowered[p.ops[P.op_end - 1].mat];
+                g = BatchProg{uint32_t(s0.lean_begin), uint32_t(s1.lean_begin + s1.lean_words - s0.lean_begin),
+                              uint32_t(P.op_end - P.op_begin), 0};
+                max_words = std::max(max_words, g.nwords);
+            }
+            progs.push_back(g);
+        }
         for (DevStage st : lowered) {
             st.sub_begin += sb_base;
             st.sub_end += sb_base;
@@ -205,6 +218,7 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     const size_t o_pass = put(h, passes), o_ops = put(h, ops), o_st = put(h, stages), o_sb = put(h, subs);
     const size_t o_circ = put(h, B->circs), o_item = put(h, B->items);
     const size_t o_words = put(h, img.words), o_pool = put(h, img.pool);
+    const size_t o_prog = put(h, progs);
     const size_t o_coef = (h.size() + 255) & ~size_t(255);
     // two spare entries: the register stages read a sub-op's first two coefficients ahead
     h.resize(o_coef + (coef.size() + 2) * amp_size(B->dt), 0);
@@ -239,6 +253,12 @@ qs_status build(qs_batch *B, int slab_bits, int stage_bits)
     a.coef = base + o_coef;
     a.words = base + o_words;
     a.pool = base + o_pool;
+    a.progs = reinterpret_cast<const BatchProg *>(base + o_prog);
+    a.max_words = max_words;
+    a.lean = lean;
+    uint64_t slabs = 0;
+    for (const BatchItem &it : B->items) slabs += it.count;
+    a.width = unsigned(slabs / std::max(1, rounds));
     a.done = static_cast<unsigned *>(B->ctl);
     a.head = a.done + B->ndone;
     a.results = reinterpret_cast<double *>(static_cast<char *>(B->ctl) +

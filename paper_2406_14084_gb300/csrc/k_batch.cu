@@ -1,4 +1,5 @@
-// k_batch.cu -- many independent circuits in one persistent launch.
+// k_batch.cu -- many independent circuits in one persistent launch (complex64 batches whose passes all
+// lower to the in-place stage engine: k_batch_lean.cu).
 //
 // The host concatenates the slab-pass plans of all circuits and lists work items (circuit,
 // pass, slab) in dependency rounds: every circuit's pass 0, then every pass 1, and so on.
@@ -17,7 +18,7 @@
 
 #include <cstdio>
 
-#include "lean_stage.cuh"
+#include "slab_common.cuh"
 
 namespace qs {
 namespace {
@@ -207,14 +208,8 @@ __global__ void __launch_bounds__(NT, 1)
             for (int o = Z.pass.op_begin; o < Z.pass.op_end; ++o) {
                 const DevOp &op = a.ops[o];
                 if ((base & op.ocmask) == op.ocmask) {
-                    if (op.type == OP_STAGE) {
-                        const DevStage *st = a.stages + op.mat;
-                        if (st->lean_begin >= 0)
-                            run_lean_stage<C, RB>(sm, GlobalWords{static_cast<const ulonglong2 *>(a.words)},
-                                                  uint32_t(st->lean_begin), static_cast<const C *>(a.pool), base, tid);
-                        else
-                            run_stage<C, RB>(sm, st, a.subs, coef, base, tid, NT);
-                    } else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
+                    if (op.type == OP_STAGE) run_stage<C, RB>(sm, a.stages + op.mat, a.subs, coef, base, tid, NT);
+                    else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
                 }
                 __syncthreads();
             }
@@ -338,6 +333,7 @@ int launch_batch_t(void *states, const BatchArgs &a, int b_max, void *stream, ch
 int launch_batch(qs_dtype dt, int stage_bits, void *states, const BatchArgs &a, int b_max, void *stream,
                  char *err, size_t errlen)
 {
+    if (a.lean) return launch_batch_lean(stage_bits, states, a, b_max, stream, err, errlen);
     if (dt == QS_C64) {
         if (stage_bits == kStageBitsC64 - 1)
             return launch_batch_t<float, kStageBitsC64 - 1, 512>(states, a, b_max, stream, err, errlen);

@@ -214,6 +214,10 @@ struct BatchItem {
     uint32_t slab;      // first slab of the run
     int32_t count;      // consecutive slabs in the run (>= 1)
 };
+// Lowered program of one pass: its words and its stages.
+struct BatchProg {
+    uint32_t begin, nwords, nstages, pad;
+};
 struct BatchTerm {
     uint64_t zm;        // physical Z mask
     double c;           // coefficient
@@ -229,6 +233,10 @@ struct BatchArgs {
     const void *coef;
     const void *words;  // lowered stages and their conditional tables
     const void *pool;
+    const BatchProg *progs;  // per pass
+    unsigned max_words;      // of the passes
+    bool lean;               // every pass has one (k_batch_lean.cu), else the general engine runs them all
+    unsigned width;          // slabs per dependency round, on average
     const BatchTerm *terms;
     unsigned *done;     // per circuit per pass: slabs stored (zeroed before each run)
     unsigned *head;     // work-queue head (zeroed before each run)
@@ -237,6 +245,8 @@ struct BatchArgs {
 };
 int launch_batch(qs_dtype dt, int stage_bits, void *states, const BatchArgs &a, int b_max, void *stream,
                  char *err, size_t errlen);
+int launch_batch_lean(int stage_bits, void *states, const BatchArgs &a, int b_max, void *stream, char *err,
+                      size_t errlen);  // complex64
 int launch_unblocked(const LaunchCtx &c, const DevOp *d_op, const DevOp &h_op,
                      const void *d_coef, char *err, size_t errlen);
 size_t pass_smem_bytes(qs_dtype dt, int b, int lo);
