@@ -73,6 +73,7 @@ struct DevPlanBuf {
     std::vector<unsigned char> h_words;
     struct Lean {             // per pass; nstages = 0: some op needs the general kernel
         int begin = 0, words = 0, stages = 0;
+        bool full = false;
     };
     std::vector<Lean> lean;
     int device = -1;
@@ -220,6 +221,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
             d.lean[i].begin = s0.lean_begin;
             d.lean[i].words = s1.lean_begin + s1.lean_words - s0.lean_begin;
             d.lean[i].stages = P.op_end - P.op_begin;
+            for (int o = P.op_begin; o < P.op_end; ++o) d.lean[i].full |= stages[p.ops[o].mat].lean_full != 0;
         }
         general = general || (!lean && P.op_begin < P.op_end);
     }
@@ -242,9 +244,9 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     const size_t o_coef = section((nc + 2) * amp_bytes(dt));
     const size_t o_cdf = section(want_df ? (nc + 2) * 16 : 0);
     const size_t o_words = section(img.words.size()), o_pool = section(img.pool.size());
-    std::vector<unsigned char> h(total, 0);
+    const std::unique_ptr<unsigned char[]> h(new unsigned char[total]);  // (padding stays unset)
     auto fill = [&](size_t off, const void *src, size_t bytes) {
-        if (bytes) std::memcpy(h.data() + off, src, bytes);
+        if (bytes) std::memcpy(h.get() + off, src, bytes);
     };
     fill(o_pass, p.passes.data(), p.passes.size() * sizeof(DevPass));
     fill(o_ops, p.ops.data(), p.ops.size() * sizeof(DevOp));
@@ -254,14 +256,16 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     fill(o_im, p.tc_images.data(), p.tc_images.size());
     fill(o_words, img.words.data(), img.words.size());
     fill(o_pool, img.pool.data(), img.pool.size());
+    std::memset(h.get() + o_coef + nc * amp_bytes(dt), 0, 2 * amp_bytes(dt));
+    if (want_df) std::memset(h.get() + o_cdf + nc * 16, 0, 32);
     if (dt == QS_C64) {
-        float *f = reinterpret_cast<float *>(h.data() + o_coef);
+        float *f = reinterpret_cast<float *>(h.get() + o_coef);
         for (size_t i = 0; i < nc; ++i) {
             f[2 * i] = (float)p.coef[i].real();
             f[2 * i + 1] = (float)p.coef[i].imag();
         }
     } else {
-        double *f = reinterpret_cast<double *>(h.data() + o_coef);
+        double *f = reinterpret_cast<double *>(h.get() + o_coef);
         for (size_t i = 0; i < nc; ++i) {
             f[2 * i] = p.coef[i].real();
             f[2 * i + 1] = p.coef[i].imag();
@@ -269,7 +273,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     }
     if (want_df) {
         // each FP64 part x as h = fl32(x), l = fl32(x - h): h + l carries about 48 bits of x
-        float *f = reinterpret_cast<float *>(h.data() + o_cdf);
+        float *f = reinterpret_cast<float *>(h.get() + o_cdf);
         for (size_t i = 0; i < nc; ++i) {
             const double parts[2] = {p.coef[i].real(), p.coef[i].imag()};
             for (int r = 0; r < 2; ++r) {
@@ -304,12 +308,12 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
             borrow->plan_ws_bytes = total;
         }
         base = borrow->plan_ws;
-        st = cuda_status(cudaMemcpyAsync(base, h.data(), total, cudaMemcpyHostToDevice, borrow->stream), "plan upload");
+        st = cuda_status(cudaMemcpyAsync(base, h.get(), total, cudaMemcpyHostToDevice, borrow->stream), "plan upload");
         if (st) return st;
     } else {
         st = cuda_status(cudaMalloc(&base, total), "plan upload allocation");
         if (st) return st;
-        st = cuda_status(cudaMemcpy(base, h.data(), total, cudaMemcpyHostToDevice), "plan upload");
+        st = cuda_status(cudaMemcpy(base, h.get(), total, cudaMemcpyHostToDevice), "plan upload");
         if (st) {
             cudaFree(base);
             return st;
@@ -394,7 +398,7 @@ qs_status run_plan(qs_state *s, qs_plan *pl, StepTimer *timer = nullptr, bool tr
             const DevPlanBuf::Lean &L = d.lean[stp.index];
             if (L.stages > 0) {
                 const LeanPassArgs la{d.h_words.data() + size_t(L.begin) * 16, (const char *)d.words + size_t(L.begin) * 16,
-                                      d.pool, L.words, L.stages, rb, d.coef_df != nullptr};
+                                      d.pool, L.words, L.stages, rb, d.coef_df != nullptr, L.full};
                 rc = launch_lean_pass(c, la, hp, err, sizeof err);
             } else {
                 // (the lowered stages of a double-float plan are in that form: not for FP64 passes)

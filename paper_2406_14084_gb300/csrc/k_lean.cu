@@ -39,7 +39,7 @@ template <> struct LeanProgram<0> {
     __device__ __forceinline__ ulonglong2 operator()(uint32_t i) const { return __ldg(g + i); }
 };
 
-template <typename R, int RB, int NT, int PER_SM, bool DF, int NW>
+template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL>
 __global__ void __launch_bounds__(NT, PER_SM)
     lean_pass_kernel(typename Cx<R>::T *__restrict__ state, const __grid_constant__ LeanProgram<NW> prog,
                      const void *__restrict__ pool, uint64_t nslabs)
@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(NT, PER_SM)
 #pragma unroll 1
         for (int o = 0; o < prog.nstages; ++o) {
             if constexpr (DF)
-                at = run_lean_stage<dfp, RB>(reinterpret_cast<dfp *>(sm), prog, at, static_cast<const dfp *>(pool), base, tid);
+                at = run_lean_stage<dfp, RB, FULL>(reinterpret_cast<dfp *>(sm), prog, at, static_cast<const dfp *>(pool), base, tid);
             else
-                at = run_lean_stage<C, RB>(sm, prog, at, static_cast<const C *>(pool), base, tid);
+                at = run_lean_stage<C, RB, FULL>(sm, prog, at, static_cast<const C *>(pool), base, tid);
             __syncthreads();
         }
 #pragma unroll 8
@@ -116,12 +116,12 @@ __global__ void __launch_bounds__(NT, PER_SM)
     }
 }
 
-template <typename R, int RB, int NT, int PER_SM, bool DF, int NW>
+template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL>
 int launch_lean_t(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h, char *err, size_t errlen)
 {
     using C = typename Cx<R>::T;
     const size_t smem = (sizeof(C) << h.b) + (sizeof(uint64_t) << h.nhi);
-    auto *const kern = lean_pass_kernel<R, RB, NT, PER_SM, DF, NW>;
+    auto *const kern = lean_pass_kernel<R, RB, NT, PER_SM, DF, NW, FULL>;
     static int attr_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -150,21 +150,23 @@ int launch_lean_t(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h, c
 
 int launch_lean_pass(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h, char *err, size_t errlen)
 {
+    constexpr int B64 = kStageBitsC64, B128 = kStageBitsC128;
     if (c.dt == QS_C64) {
-        if (a.stage_bits == kStageBitsC64 - 1)
-            return launch_lean_t<float, kStageBitsC64 - 1, 512, 1, false, 0>(c, a, h, err, errlen);
-        if (a.nwords <= 480) return launch_lean_t<float, kStageBitsC64, 256, 2, false, 480>(c, a, h, err, errlen);
-        if (a.nwords <= 2000) return launch_lean_t<float, kStageBitsC64, 256, 2, false, 2000>(c, a, h, err, errlen);
-        return launch_lean_t<float, kStageBitsC64, 256, 2, false, 0>(c, a, h, err, errlen);
+        if (a.stage_bits == B64 - 1) return launch_lean_t<float, B64 - 1, 512, 1, false, 0, true>(c, a, h, err, errlen);
+        if (a.nwords > 2000) return launch_lean_t<float, B64, 256, 2, false, 0, true>(c, a, h, err, errlen);
+        if (a.full)
+            return a.nwords <= 480 ? launch_lean_t<float, B64, 256, 2, false, 480, true>(c, a, h, err, errlen)
+                                   : launch_lean_t<float, B64, 256, 2, false, 2000, true>(c, a, h, err, errlen);
+        return a.nwords <= 480 ? launch_lean_t<float, B64, 256, 2, false, 480, false>(c, a, h, err, errlen)
+                               : launch_lean_t<float, B64, 256, 2, false, 2000, false>(c, a, h, err, errlen);
     }
     if (a.df) {
-        if (a.stage_bits == kStageBitsC128 - 1)
-            return launch_lean_t<double, kStageBitsC128 - 1, 512, 1, true, 0>(c, a, h, err, errlen);
-        return launch_lean_t<double, kStageBitsC128, 256, 2, true, 0>(c, a, h, err, errlen);
+        if (a.stage_bits == B128 - 1) return launch_lean_t<double, B128 - 1, 512, 1, true, 0, true>(c, a, h, err, errlen);
+        return a.full ? launch_lean_t<double, B128, 256, 2, true, 0, true>(c, a, h, err, errlen)
+                      : launch_lean_t<double, B128, 256, 2, true, 0, false>(c, a, h, err, errlen);
     }
-    if (a.stage_bits == kStageBitsC128 - 1)
-        return launch_lean_t<double, kStageBitsC128 - 1, 512, 1, false, 0>(c, a, h, err, errlen);
-    return launch_lean_t<double, kStageBitsC128, 256, 2, false, 0>(c, a, h, err, errlen);
+    if (a.stage_bits == B128 - 1) return launch_lean_t<double, B128 - 1, 512, 1, false, 0, true>(c, a, h, err, errlen);
+    return launch_lean_t<double, B128, 256, 2, false, 0, true>(c, a, h, err, errlen);
 }
 
 }  // namespace qs

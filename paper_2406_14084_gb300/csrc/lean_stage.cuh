@@ -92,10 +92,10 @@ __device__ __forceinline__ void for_half(F &&f)
     for (int e = 0; e < (1 << RB); ++e)
         if ((e >> J & 1) == V) f(e);
 }
-template <int RB, typename F>
+template <int RB, bool HALVES, typename F>
 __device__ __forceinline__ void for_pattern(uint32_t pat, F &&f)
 {
-    switch (pat) {
+    switch (HALVES ? pat : 0u) {
     case 1: for_half<RB, 0, 0>(f); break;
     case 2: for_half<RB, 0, 1>(f); break;
     case 3: for_half<RB, 1, 0>(f); break;
@@ -189,15 +189,52 @@ template <int RB> struct LeanRegs<float2, RB> {
         }
     }
     // word p: both real parts, both imaginary parts of the factors of pair p
-    template <typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t /*pat*/)
+    template <bool HALVES, typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t pat)
     {
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
+        // (patterns of register bit 0, inside the pairs, are not used here)
+        for_pattern<RB - 1, HALVES>(pat > 2 ? pat - 2 : 0, [&](int p) {
             const ulonglong2 q = words.bulk(at + (uint32_t(p) << nl));
-            const unsigned long long m = mul2(q.y ^ 0x8000000080000000ull, Y[p]), w = mul2(q.y, X[p]);
-            X[p] = fma2(q.x, X[p], m);
-            Y[p] = fma2(q.x, Y[p], w);
+            times(p, q.x, q.y);
+        });
+    }
+    // pair p times (re, im), each for both elements
+    __device__ __forceinline__ void times(int p, unsigned long long re, unsigned long long im)
+    {
+        const unsigned long long m = mul2(im ^ 0x8000000080000000ull, Y[p]), w = mul2(im, X[p]);
+        X[p] = fma2(re, X[p], m);
+        Y[p] = fma2(re, Y[p], w);
+    }
+    // separable table: f[0] = s, f[1 + j] = phi_j
+    struct Sep {
+        float2 f[RB + 1];
+        template <typename W> __device__ __forceinline__ void group(const W &words, uint32_t at, uint32_t nl, bool first)
+        {
+#pragma unroll
+            for (int k = 0; k <= RB; k += 2) {
+                const ulonglong2 q = words.bulk(at + (uint32_t(k >> 1) << nl));
+                const float2 a = unpack2(q.x), b = unpack2(q.y);
+                f[k] = first ? a : cmul(a, f[k]);
+                if (k + 1 <= RB) f[k + 1] = first ? b : cmul(b, f[k + 1]);
+            }
         }
+    };
+    static constexpr int kSepWords = (RB + 2) / 2;
+    // the factors of the pairs come from a walk over the register bits, one multiply per step down
+    template <int BIT> __device__ __forceinline__ void sep_walk(const Sep &t, int p, unsigned long long re, unsigned long long im)
+    {
+        if constexpr (BIT == RB - 1) {
+            times(p, re, im);
+        } else {
+            sep_walk<BIT + 1>(t, p, re, im);
+            const float2 g = t.f[BIT + 2];
+            const unsigned long long gx = pack2(g.x, g.x), gy = pack2(g.y, g.y), ny = pack2(-g.y, -g.y);
+            sep_walk<BIT + 1>(t, p | (1 << BIT), fma2(gx, re, mul2(ny, im)), fma2(gx, im, mul2(gy, re)));
+        }
+    }
+    template <bool ONE> __device__ __forceinline__ void sep(const Sep &t)
+    {
+        const float2 u = cmul(t.f[0], t.f[1]);
+        sep_walk<0>(t, 0, pack2(t.f[0].x, u.x), pack2(t.f[0].y, u.y));
     }
     template <typename W> __device__ __forceinline__ void scale(const W &words, uint32_t at)
     {
@@ -309,10 +346,33 @@ template <int RB> struct LeanRegs<double2, RB> {
         return make_double2(__longlong_as_double((long long)w.x), __longlong_as_double((long long)w.y));
     }
     // elements outside the pattern have the factor 1
-    template <typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t pat)
+    template <bool HALVES, typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t pat)
     {
-        for_pattern<RB>(pat, [&](int e) { v[e] = cmul(factor(words(at + (uint32_t(e) << nl))), v[e]); });
+        for_pattern<RB, HALVES>(pat, [&](int e) { v[e] = cmul(factor(words(at + (uint32_t(e) << nl))), v[e]); });
     }
+    struct Sep {
+        C f[RB + 1];
+        template <typename W> __device__ __forceinline__ void group(const W &words, uint32_t at, uint32_t nl, bool first)
+        {
+#pragma unroll
+            for (int k = 0; k <= RB; ++k) {
+                const C a = factor(words(at + (uint32_t(k) << nl)));
+                f[k] = first ? a : cmul(a, f[k]);
+            }
+        }
+    };
+    static constexpr int kSepWords = RB + 1;
+    // ONE: the factor so far is 1
+    template <int BIT, bool ONE> __device__ __forceinline__ void sep_walk(const Sep &t, int e, C f)
+    {
+        if constexpr (BIT == RB) {
+            if (!ONE) v[e] = cmul(f, v[e]);
+        } else {
+            sep_walk<BIT + 1, ONE>(t, e, f);
+            sep_walk<BIT + 1, false>(t, e | (1 << BIT), ONE ? t.f[BIT + 1] : cmul(t.f[BIT + 1], f));
+        }
+    }
+    template <bool ONE> __device__ __forceinline__ void sep(const Sep &t) { sep_walk<0, ONE>(t, 0, t.f[0]); }
     template <typename W> __device__ __forceinline__ void scale(const W &words, uint32_t at)
     {
 #pragma unroll
@@ -332,7 +392,7 @@ template <int RB> struct LeanRegs<double2, RB> {
     {
         if (!on) return;
         const C t = factor(w);
-        for_pattern<RB>(pat, [&](int e) {
+        for_pattern<RB, true>(pat, [&](int e) {
             const bool in = elems >> e & 1u;
             v[e] = cmul(make_double2(in ? t.x : 1.0, in ? t.y : 0.0), v[e]);
         });
@@ -450,10 +510,41 @@ template <int RB> struct LeanRegs<dfp, RB> {
         w.l = pack2(l.y, l.x);
         v = df_fma(df_factor(t.x, t.y), v, df_mul(df_factor(pack2(-t.z, t.z), pack2(-t.w, t.w)), w));
     }
-    template <typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t pat)
+    template <bool HALVES, typename W> __device__ __forceinline__ void table(const W &words, uint32_t at, uint32_t nl, uint32_t pat)
     {
-        for_pattern<RB>(pat, [&](int e) { times(v[e], factor(words(at + (uint32_t(e) << nl)))); });
+        for_pattern<RB, HALVES>(pat, [&](int e) { times(v[e], factor(words(at + (uint32_t(e) << nl)))); });
     }
+    static __device__ __forceinline__ dfp as_dfp(float4 t) { return dfp{pack2(t.x, t.z), pack2(t.y, t.w)}; }
+    static __device__ __forceinline__ float4 as_factor(const dfp &a)
+    {
+        const float2 h = unpack2(a.h), l = unpack2(a.l);
+        return make_float4(h.x, l.x, h.y, l.y);
+    }
+    struct Sep {
+        dfp f[RB + 1];
+        template <typename W> __device__ __forceinline__ void group(const W &words, uint32_t at, uint32_t nl, bool first)
+        {
+#pragma unroll
+            for (int k = 0; k <= RB; ++k) {
+                const float4 a = factor(words(at + (uint32_t(k) << nl)));
+                if (first) f[k] = as_dfp(a);
+                else times(f[k], a);
+            }
+        }
+    };
+    static constexpr int kSepWords = RB + 1;
+    template <int BIT, bool ONE> __device__ __forceinline__ void sep_walk(const Sep &t, int e, dfp f)
+    {
+        if constexpr (BIT == RB) {
+            if (!ONE) times(v[e], as_factor(f));
+        } else {
+            sep_walk<BIT + 1, ONE>(t, e, f);
+            dfp g = t.f[BIT + 1];
+            if (!ONE) times(g, as_factor(f));
+            sep_walk<BIT + 1, false>(t, e | (1 << BIT), g);
+        }
+    }
+    template <bool ONE> __device__ __forceinline__ void sep(const Sep &t) { sep_walk<0, ONE>(t, 0, t.f[0]); }
     template <typename W> __device__ __forceinline__ void scale(const W &words, uint32_t at)
     {
 #pragma unroll
@@ -476,7 +567,7 @@ template <int RB> struct LeanRegs<dfp, RB> {
     {
         if (!on) return;
         const float4 t = factor(w);
-        for_pattern<RB>(pat, [&](int e) {
+        for_pattern<RB, true>(pat, [&](int e) {
             const bool in = elems >> e & 1u;
             times(v[e], make_float4(in ? t.x : 1.f, in ? t.y : 0.f, in ? t.z : 0.f, in ? t.w : 0.f));
         });
@@ -539,12 +630,25 @@ __device__ __forceinline__ uint4 as_u4(ulonglong2 w)
     return make_uint4(uint32_t(w.x), uint32_t(w.x >> 32), uint32_t(w.y), uint32_t(w.y >> 32));
 }
 
+// Values of a record's condition bits: x = those inside the slab (nl of them), y = those outside it,
+// which are the same for the whole slab.
+__device__ __forceinline__ uint2 condition_index(ulonglong2 cw, uint32_t nl, uint32_t ndl, uint32_t base, uint64_t cta_base)
+{
+    unsigned long long codes = cw.x;
+    uint32_t hl = 0, ho = 0, k = 0;
+    for (; k < nl; ++k, codes = k == 8 ? cw.y : codes >> 8) hl |= ((base >> (codes & 0x7fu)) & 1u) << k;
+    for (; k < ndl; ++k, codes = k == 8 ? cw.y : codes >> 8) ho |= uint32_t((cta_base >> (codes & 0x7fu)) & 1u) << (k - nl);
+    return make_uint2(hl, ho);
+}
+
 // Runs the stage whose words start at `at` on the slab in shared memory (addressing: run_stage) and
 // returns the index after its last word.  One group per thread, the caller has at least 2^nrest threads.
 // (With a loop over groups the compiler keeps the 31 address offsets live across it, which costs
 // spills at 128 registers.)  Threads without a group work on a copy of one and store nothing, so that
 // control flow stays the same for the whole warp.
-template <typename C, int RB, typename Words>
+// FULL = false: stages without separable tables, X and half tables, in complex64 without phases too.  The larger set
+// costs the common records registers and moves (layered-28 complex64: 41.2 ms with one set, 37.8 with two).
+template <typename C, int RB, bool FULL = true, typename Words>
 __device__ __forceinline__ uint32_t run_lean_stage(C *sm, const Words &words, uint32_t at, const C *__restrict__ pool,
                                                    uint64_t cta_base, uint32_t tid)
 {
@@ -590,22 +694,32 @@ __device__ __forceinline__ uint32_t run_lean_stage(C *sm, const Words &words, ui
         case L_ROTM2: if constexpr (PL == 0) v.template rot<2, true>(words, at); at += V::kRotWords; break;
         case L_ROTM3: if constexpr (PL == 0 && RB > 3) v.template rot<3, true>(words, at); at += V::kRotWords; break;
         case L_CONST:  // a table without conditions: its factors follow
-            v.table(words, at + 1, 0, h.z);
+            v.template table<FULL>(words, at + 1, 0, h.z);
             at += 1 + V::kConstWords;
             break;
         case L_TABLE: {
-            // nl conditions inside the slab, then those outside it (the same for the whole slab)
-            const uint32_t nl = (h.x >> 16) & 0xffu, ndl = h.x >> 24;
-            const ulonglong2 cw = words(at + 1);
-            unsigned long long codes = cw.x;
-            uint32_t hl = 0, ho = 0, k = 0;
-            for (; k < nl; ++k, codes = k == 8 ? cw.y : codes >> 8) hl |= ((base >> (codes & 0x7fu)) & 1u) << k;
-            for (; k < ndl; ++k, codes = k == 8 ? cw.y : codes >> 8)
-                ho |= uint32_t((cta_base >> (codes & 0x7fu)) & 1u) << (k - nl);
-            v.table(GlobalWords{reinterpret_cast<const ulonglong2 *>(pool) + (h.y + (ho << (RB - PL + nl)) + hl)}, 0, nl, h.z);
+            const uint32_t nl = (h.x >> 16) & 0xffu;
+            const uint2 i = condition_index(words(at + 1), nl, h.x >> 24, base, cta_base);
+            v.template table<FULL>(GlobalWords{reinterpret_cast<const ulonglong2 *>(pool) + (h.y + (i.y << (RB - PL + nl)) + i.x)}, 0, nl, h.z);
             at += 2;
             break;
         }
+        case L_SEP:
+        case L_SEP1: if constexpr (FULL) {
+            typename V::Sep t;
+            const uint32_t ng = (h.x >> 8) & 0xffu;
+            for (uint32_t g = 0; g < ng; ++g) {
+                const uint4 gw = as_u4(words(at + 1 + 2 * g));
+                const uint32_t nl = gw.y & 0xffu;
+                const uint2 i = condition_index(words(at + 2 + 2 * g), nl, (gw.y >> 8) & 0xffu, base, cta_base);
+                t.group(GlobalWords{reinterpret_cast<const ulonglong2 *>(pool) + (gw.x + ((i.y * V::kSepWords) << nl) + i.x)}, 0,
+                        nl, g == 0);
+            }
+            if ((h.x & 0xffu) == L_SEP) v.template sep<false>(t);
+            else v.template sep<true>(t);
+            at += 1 + 2 * ng;
+        }
+            break;
         case L_SCALE:
             v.scale(words, at + 1);
             at += 1 + V::kScaleWords;
@@ -615,7 +729,7 @@ __device__ __forceinline__ uint32_t run_lean_stage(C *sm, const Words &words, ui
             const uint4 c = as_u4(words(at + 1));  // conditions
             const uint64_t ocm = uint64_t(c.w) << 32 | c.z;
             const bool on = (base & c.x) == c.x && (cta_base & ocm) == ocm;
-            if ((h.x & 0xffu) == L_SIGN) {
+            if ((!FULL && PL == 1) || (h.x & 0xffu) == L_SIGN) {
                 v.sign(on ? h.y : 0u);
                 at += 2;
             } else {
@@ -624,7 +738,7 @@ __device__ __forceinline__ uint32_t run_lean_stage(C *sm, const Words &words, ui
             }
             break;
         }
-        default: {  // L_CX
+        default: if constexpr (FULL) {  // L_CX
             const uint4 c = as_u4(words(at + 1));
             const uint64_t ocm = uint64_t(c.w) << 32 | c.z;
             const uint32_t m = ((base & c.x) == c.x && (cta_base & ocm) == ocm) ? ~0u : 0u;
@@ -638,8 +752,8 @@ __device__ __forceinline__ uint32_t run_lean_stage(C *sm, const Words &words, ui
             default: break;
             }
             at += 2;
-            break;
         }
+            break;
         }
     }
     if (mine) {

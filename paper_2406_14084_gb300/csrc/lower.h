@@ -8,6 +8,13 @@
 
 namespace qs {
 
+// One group of a separable table: factor(e) = s prod_j phi_j^(e_j), with s and phi looked up by the
+// condition bits dl: entry h (RB + 1) + 0 is s, + 1 + j is phi_j.
+struct SepGroup {
+    std::vector<uint8_t> dl;
+    std::vector<cd> tab;
+};
+
 // One record of a lowered stage, in FP64; lower_stages() writes it in the state precision.
 struct LeanItem {
     LeanOp op = L_ROTA;
@@ -19,6 +26,7 @@ struct LeanItem {
     uint32_t neg = 0;
     std::vector<cd> tab;            // L_TABLE: 2^(RB + ndl) factors, index (hi << RB) | e
     std::vector<uint8_t> dl;        // L_TABLE: condition bits (DevSub::dl codes)
+    std::vector<SepGroup> sep;      // L_SEP
     std::vector<double> scale;      // L_SCALE: 2^RB real factors
     uint32_t rd = 0;                // diagonals: register bits the factors may depend on
     uint32_t m32 = 0;               // L_PHASE: register elements the phase p acts on

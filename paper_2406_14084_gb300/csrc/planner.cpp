@@ -1047,6 +1047,9 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
             plan.subs.push_back(s);
         }
         factor_stage_rotations(plan, st.sub_begin, cf);
+        plan.raw_range.emplace_back((int)plan.raw_subs.size(), 0);
+        plan.raw_subs.insert(plan.raw_subs.end(), plan.subs.begin() + st.sub_begin, plan.subs.end());
+        plan.raw_range.back().second = (int)plan.raw_subs.size();
         merge_stage_diagonals(plan, st.sub_begin, RB, cf);
         st.sub_end = (int)plan.subs.size();
         DevOp op;

@@ -3,6 +3,7 @@
 
 #include <complex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "qs_internal.h"
@@ -47,6 +48,9 @@ struct Plan {
     std::vector<DevOp> ops;
     std::vector<DevStage> stages;
     std::vector<DevSub> subs;
+    // sub-ops of each stage before its diagonals were merged into tables (lower.cpp regroups them)
+    std::vector<DevSub> raw_subs;
+    std::vector<std::pair<int, int>> raw_range;  // per stage
     std::vector<DevTc> tcs;                 // tensor-core steps
     std::vector<unsigned char> tc_images;   // their E_hi / E_lo operand images
     std::vector<uint32_t> tc_coef;          // FP64 matrix of each tensor-core step (for listings)

@@ -101,7 +101,7 @@ struct alignas(16) DevSub {
 };
 static_assert(sizeof(DevSub) == 48, "DevSub layout");
 
-struct DevStage {
+struct alignas(8) DevStage {
     uint8_t r;          // register bits
     uint8_t nrest;      // non-register slab-local bits
     uint8_t sbits[6];   // slab-local position of register bit j
@@ -111,7 +111,10 @@ struct DevStage {
     // the stage for the in-place engine (lower.cpp, lean_stage.cuh): its first 16-byte word, or
     // lean_begin < 0 where the stage holds a sub-op that only the general engine runs
     int32_t lean_begin, lean_words;
+    int32_t lean_full;  // it holds a separable or half table, a phase or an X
+    int32_t pad;
 };
+static_assert(sizeof(DevStage) % 8 == 0, "DevStage is read with 8-byte loads");
 
 // Words of a lowered stage.  Head: {u8 register bit positions[RB] (8 bytes), u32 nrest | flip << 8,
 // u32 number of words that follow}; flip: register bits whose two values the stage exchanges when it
@@ -128,6 +131,10 @@ enum LeanOp : uint8_t {
     L_CONST,      // u32 at byte 8 = pattern that holds the factors other than 1; all factors follow
     L_TABLE,      // arg = first word in the pool; byte 8 as L_CONST; ndl condition bits, the first b of
                   // them inside the slab; a word of condition codes u8[12] (as DevSub::dl)
+    L_SEP,        // a = groups; per group a word {u32 first word in the pool, u8 nl, u8 ndl} and a word of
+                  // condition codes.  The factor of element e is the product over the groups of
+                  // s prod_j phi_j^(e_j); a group holds (s, phi_0, ..) per setting of its conditions
+    L_SEP1,       // the same with s = 1 throughout
     L_SCALE,      // real factors follow
     L_SIGN,       // arg = elements whose sign changes; conditions
     L_PHASE,      // arg = elements; byte 8 = pattern that holds them; conditions; the factor
@@ -188,6 +195,7 @@ struct LeanPassArgs {
     const void *h_words, *d_words, *pool;
     int nwords, nstages, stage_bits;
     bool df;
+    bool full;  // some record is outside the plain set (DevStage::lean_full)
 };
 int launch_lean_pass(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h_pass, char *err, size_t errlen);
 int launch_pass(const LaunchCtx &c, const PassArgs &a, const DevPass &h_pass, char *err,

@@ -77,3 +77,10 @@ def test_conditional_tables(merge, dtype, arith, tol):
 def test_program_sizes(depth):
     """One pass of a 13-qubit state: words in 8 KB and 32 KB of parameters, then in device memory."""
     check(13, W.layered(13, depth, 11), qs.QS_C64, 1e-5)
+
+
+@pytest.mark.parametrize("dtype,arith,tol", FORMS)
+@pytest.mark.parametrize("n,slab", [(8, 0), (14, 0), (15, 7), (17, 11)])
+def test_separable_tables(n, slab, dtype, arith, tol):
+    """Many conditional phases at one place: condition groups inside the slab, outside it and in both."""
+    check(n, W.qaoa_complete(n, 2, 3 + n) + W.qft(n), dtype, tol, slab_bits=slab, arith=arith)
