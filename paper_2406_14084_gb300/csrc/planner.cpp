@@ -1574,6 +1574,35 @@ int build_plan(const std::vector<CGate> &gates_in, int n, qs_dtype dt, const qs_
                 note_skipped(roles[i], skipped);
             }
         }
+        // Diagonals that no later op of this pass waits for go to the pass (and there to the stage) that
+        // needs them: they then meet the diagonals of the next layer in one table.  (qft28 complex128
+        // 76.6 -> 72.2 ms, qaoa23 complex64 575 -> 529 us, layered25 complex128 95.8 -> 94.8 ms.  Where
+        // only single-qubit ones would go it is left: they only grow a table there, and their pass needs
+        // a scaling for the factors its table had taken.)
+        bool more = !tc;
+        if (more) {
+            more = false;
+            for (size_t i = first; i < gates.size() && !more; ++i) more = !done[i] && gates[i].cls != C_DIAG;
+        }
+        if (more) {
+            std::vector<char> keep(sched.size(), 1);
+            uint64_t waits = 0;  // qubits that a later op of the pass acts on non-diagonally
+            bool joint = false;  // single-qubit ones alone meet nothing there
+            for (size_t k = sched.size(); k-- > 0;) {
+                const int i = sched[k].gate;
+                if (gates[i].cls == C_DIAG && !(roles[i].any & waits)) {
+                    keep[k] = 0;
+                    joint |= (roles[i].any & (roles[i].any - 1)) != 0;
+                }
+                waits |= roles[i].nondiag;
+            }
+            if (waits && joint)
+                for (size_t k = sched.size(); k-- > 0;)
+                    if (!keep[k]) {
+                        done[sched[k].gate] = 0;
+                        sched.erase(sched.begin() + k);
+                    }
+        }
         if (!sched.empty()) {
             emit_pass(plan, gates, S, lo, b, n, sched, S_PASS, dt);
             stalls = 0;
