@@ -11,7 +11,9 @@
 // the parity of j & z splits into a part of the thread and a part of k that the whole grid shares.
 // Bound by shared-memory reads (one amplitude pair per mask) and FP32 / FP64 issue, no longer by HBM:
 // a Heisenberg chain of 26 qubits (25 bond masks, 75 terms, and the field) took 14.6 ms with one pass
-// per mask and takes 1.76 ms.
+// per mask and takes 1.27 ms (24 qubits in complex128: 2.03).  Three CTAs fit an SM (64 KiB of tile each,
+// terms and offsets behind it as many as there are: two CTAs 1.76 ms, three 1.37); terms whose sign is the
+// same for all pairs of a thread, most of a chain's, share one sum (1.37 -> 1.27 ms, complex128 2.99 -> 2.03).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -53,7 +55,7 @@ __device__ __forceinline__ double with_sign(double v, uint32_t s)
 }
 
 template <typename R>
-__global__ void __launch_bounds__(kThreads) pauli_tile_kernel(const typename Cx<R>::T *__restrict__ a, int b,
+__global__ void __launch_bounds__(kThreads, 3) pauli_tile_kernel(const typename Cx<R>::T *__restrict__ a, int b,
                                                               const PauliTile *__restrict__ d, uint64_t ntiles,
                                                               double *__restrict__ part)
 {
@@ -61,12 +63,13 @@ __global__ void __launch_bounds__(kThreads) pauli_tile_kernel(const typename Cx<
     constexpr int K = 1 << (tile_bits<R>() - 9);  // pairs per thread of a full tile
     extern __shared__ __align__(16) unsigned char dyn[];
     C *const sm = reinterpret_cast<C *>(dyn);
-    __shared__ uint64_t seg[512];
-    __shared__ PauliGroup G[kMaxGroups];
-    __shared__ PauliTerm T[kMaxTerms];
     __shared__ double red[kThreads / 32];
     const uint32_t tid = threadIdx.x;
     const int lo = d->lo, nhi = d->nhi, ng = d->ngroups, nt = d->nterms;
+    // [tile][segment offsets][terms][groups]
+    uint64_t *const seg = reinterpret_cast<uint64_t *>(sm + (size_t(1) << b));
+    PauliTerm *const T = reinterpret_cast<PauliTerm *>(seg + (size_t(1) << nhi));
+    PauliGroup *const G = reinterpret_cast<PauliGroup *>(T + nt);
     for (uint32_t s = tid; s < (1u << nhi); s += kThreads) {
         uint64_t o = 0;
         for (int m = 0; m < nhi; ++m)
@@ -98,37 +101,51 @@ __global__ void __launch_bounds__(kThreads) pauli_tile_kernel(const typename Cx<
         for (int g = 0; g < ng; ++g) {
             const PauliGroup q = G[g];
             const uint32_t low = (1u << q.piv) - 1;
-            R vr[K], vi[K];
+            R v[K];
+            auto terms = [&](int from, int to) {
+                // (terms without a sign inside a thread share the plain sum)
+                R p0 = 0, p1 = 0;
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const uint32_t j = tid + uint32_t(k) * kThreads;
-                vr[k] = vi[k] = R(0);
-                if (j < pairs) {
-                    const uint32_t i0 = ((j & ~low) << 1) | (j & low);
-                    const C x = sm[i0], y = sm[i0 ^ q.xm];
-                    vr[k] = y.x * x.x + y.y * x.y;
-                    vi[k] = y.x * x.y - y.y * x.x;
+                for (int k = 0; k < K; k += 2) {
+                    p0 += v[k];
+                    p1 += v[k + 1];
                 }
+                for (int t = from; t < to; ++t) {
+                    const uint32_t odd = (__popcll(base & T[t].zout) + __popc(tid & T[t].zthr)) & 1u;
+                    const uint32_t kp = T[t].kpat;
+                    R s = p0 + p1;
+                    if (kp) {
+                        R s0 = 0, s1 = 0;
+#pragma unroll
+                        for (int k = 0; k < K; k += 2) {
+                            s0 += with_sign(v[k], (kp << (31 - k)) & 0x80000000u);
+                            s1 += with_sign(v[k + 1], (kp << (30 - k)) & 0x80000000u);
+                        }
+                        s = s0 + s1;
+                    }
+                    const R c = (R)T[t].c;
+                    facc = fma(odd ? -c : c, s, facc);
+                }
+            };
+            auto values = [&](bool imag) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const uint32_t j = tid + uint32_t(k) * kThreads;
+                    v[k] = R(0);
+                    if (j < pairs) {
+                        const uint32_t i0 = ((j & ~low) << 1) | (j & low);
+                        const C x = sm[i0], y = sm[i0 ^ q.xm];
+                        v[k] = imag ? y.x * x.y - y.y * x.x : y.x * x.x + y.y * x.y;
+                    }
+                }
+            };
+            if (q.t0 < q.tmid) {
+                values(false);
+                terms(q.t0, q.tmid);
             }
-            for (int t = q.t0; t < q.t1; ++t) {
-                const uint32_t odd = (__popcll(base & T[t].zout) + __popc(tid & T[t].zthr)) & 1u;
-                const uint32_t kp = T[t].kpat;
-                R s0 = 0, s1 = 0;
-                if (t < q.tmid) {
-#pragma unroll
-                    for (int k = 0; k < K; k += 2) {
-                        s0 += with_sign(vr[k], (kp << (31 - k)) & 0x80000000u);
-                        s1 += with_sign(vr[k + 1], (kp << (30 - k)) & 0x80000000u);
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < K; k += 2) {
-                        s0 += with_sign(vi[k], (kp << (31 - k)) & 0x80000000u);
-                        s1 += with_sign(vi[k + 1], (kp << (30 - k)) & 0x80000000u);
-                    }
-                }
-                const R c = (R)T[t].c;
-                facc = fma(odd ? -c : c, s0 + s1, facc);
+            if (q.tmid < q.t1) {
+                values(true);
+                terms(q.tmid, q.t1);
             }
         }
         acc += (double)facc;
@@ -147,19 +164,21 @@ __global__ void __launch_bounds__(kThreads) pauli_tile_kernel(const typename Cx<
 }
 
 template <typename R>
-int launch_t(const LaunchCtx &c, const PauliTile *d, int b, double *part, int max_blocks)
+int launch_t(const LaunchCtx &c, const PauliTile *d, const PauliTile &h, int b, double *part, int max_blocks)
 {
     using C = typename Cx<R>::T;
-    const size_t smem = sizeof(C) << b;
+    const size_t smem = (sizeof(C) << b) + (sizeof(uint64_t) << h.nhi) + h.nterms * sizeof(PauliTerm) +
+                        h.ngroups * sizeof(PauliGroup);
     static int attr_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
     if (attr_dev != dev) {
-        cudaFuncSetAttribute(pauli_tile_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+        cudaFuncSetAttribute(pauli_tile_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int((64 << 10) + (8 << 9) + kMaxTerms * sizeof(PauliTerm) + kMaxGroups * sizeof(PauliGroup)));
         attr_dev = dev;
     }
     const uint64_t ntiles = 1ull << (c.n - b);
-    const uint64_t per_sm = smem >= 64 * 1024 ? 2 : 4;
+    const uint64_t per_sm = 3 * (smem + 1088) <= 228 * 1024 ? 3 : 2;  // (with the block's own shared memory and reserve)
     const int blocks = int(std::min<uint64_t>({ntiles, uint64_t(num_sms()) * per_sm, uint64_t(max_blocks)}));
     pauli_tile_kernel<R><<<blocks, kThreads, smem, (cudaStream_t)c.stream>>>(reinterpret_cast<const C *>(c.amp), b, d, ntiles,
                                                                              part);
@@ -240,10 +259,11 @@ int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, 
     return b;
 }
 
-int launch_pauli_tile(const LaunchCtx &c, const void *d_tile, int b, double *part, int max_blocks)
+int launch_pauli_tile(const LaunchCtx &c, const void *d_tile, const void *h_tile, int b, double *part, int max_blocks)
 {
     const PauliTile *d = static_cast<const PauliTile *>(d_tile);
-    return c.dt == QS_C64 ? launch_t<float>(c, d, b, part, max_blocks) : launch_t<double>(c, d, b, part, max_blocks);
+    const PauliTile &h = *static_cast<const PauliTile *>(h_tile);
+    return c.dt == QS_C64 ? launch_t<float>(c, d, h, b, part, max_blocks) : launch_t<double>(c, d, h, b, part, max_blocks);
 }
 
 }  // namespace qs

@@ -665,7 +665,7 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
         for (int g : tiles) done[g] = 0;
         if (cudaMemcpyAsync(dtile, htile.data(), htile.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
             return cuda_fail("expect upload", err, errlen);
-        const int nblk = launch_pauli_tile(c, dtile, b, part, kRedBlocksMax);
+        const int nblk = launch_pauli_tile(c, dtile, htile.data(), b, part, kRedBlocksMax);
         finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
         int rc = cuda_fail("expect launch", err, errlen);
         if (rc) return rc;
