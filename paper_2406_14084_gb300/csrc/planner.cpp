@@ -892,7 +892,12 @@ void build_stages(Plan &plan, const std::vector<CGate> &gates, const std::vector
             switch (g.cls) {
             case C_DENSE: r = g.tq.size() <= 2; break;
             case C_PERMX: case C_SWAP: r = true; break;
-            case C_DIAG: r = controlled_phase(g, ph0) || (g.tq.size() + g.cq.size() <= 7); break;
+            case C_DIAG:
+                // As an op of its own a fused table of 8-10 qubits sent the whole pass to the general kernel
+                // (random20 complex128 818 -> 790 us).  A table grows to 2^RB factors per setting of its bits
+                // outside the registers: up to ten it is no larger than the merged ones.
+                r = controlled_phase(g, ph0) || g.tq.size() + g.cq.size() <= 10;
+                break;
             }
         }
         regable[i] = r;

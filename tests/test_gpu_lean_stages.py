@@ -84,3 +84,17 @@ def test_program_sizes(depth):
 def test_separable_tables(n, slab, dtype, arith, tol):
     """Many conditional phases at one place: condition groups inside the slab, outside it and in both."""
     check(n, W.qaoa_complete(n, 2, 3 + n) + W.qft(n), dtype, tol, slab_bits=slab, arith=arith)
+
+
+@pytest.mark.parametrize("dtype,arith,tol", FORMS)
+@pytest.mark.parametrize("k", [7, 8, 10, 11])
+def test_wide_diagonals(k, dtype, arith, tol):
+    """Diagonals of up to eleven qubits, controls included (ten: the widest that stages take), between rotations, with bits inside and outside the slab."""
+    n = 14
+    rng = W.SplitMix64(300 + k)
+    tables = []
+    for i in range(2):
+        q = tuple(rng.distinct(n, k))
+        tables.append(Gate("DIAG", q[:7], q[7:], (), W.random_diag(7, 70 + i)))
+    check(n, mixed(n, 30, k) + tables[:1] + mixed(n, 30, 90 + k) + tables[1:] + mixed(n, 20, 50 + k), dtype, tol, slab_bits=9,
+          arith=arith)
