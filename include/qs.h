@@ -141,8 +141,9 @@ typedef struct {
     int32_t input_gates;   /* gates given to qs_fuse */
     int32_t slab_bits, seg_bits;
     double flops_per_amp;  /* modelled arithmetic per amplitude, summed over the plan */
-    int64_t device_bytes;  /* bytes the plan uploads to the device (descriptors + coefficients)
-                              for a complex128 state; half the coefficient bytes for complex64 */
+    int64_t device_bytes;  /* size of the plan's descriptors and coefficients for a complex128 state
+                              (complex64: half the coefficient bytes); register stages are
+                              uploaded as programs and tables made from them */
     int32_t stages;        /* register stages over all passes */
     int32_t stage_ops;     /* ops executed inside register stages */
     int32_t smem_ops;      /* ops executed directly on the shared-memory slab */
@@ -290,9 +291,10 @@ qs_status qs_probs_noalloc(const void *dev_amp, int n, qs_dtype dt, const int *q
 qs_status qs_sample(qs_state *s, const double *u, size_t shots, uint64_t *host_out);
 
 /* host_out[0] = Re sum_t coeff_t <psi|P_t|psi>, host_out[1] = its imaginary part (zero up to
- * rounding for Hermitian sums).  Terms are grouped by X mask (at most 256 per group) and each
- * group costs one read of the state; groups of four or more terms on 16 or more qubits go
- * through Walsh-Hadamard tiles, so that read costs the same whatever the group's size.  FP64
+ * rounding for Hermitian sums).  Terms are grouped by X mask (at most 256 per group).  Groups of four
+ * or more terms on 16 or more qubits cost one read of the state each, through Walsh-Hadamard
+ * tiles, whatever the group's size; smaller groups share reads where their X masks fit the bits of
+ * one shared-memory tile (13 qubits, complex128 12), and take one read each otherwise.  FP64
  * accumulation across tiles (complex64 states: FP32 within a tile).  Synchronises. */
 qs_status qs_expect_pauli_sum(qs_state *s, const qs_pauli_term *terms, size_t nterms,
                               double *host_out);
