@@ -11,7 +11,7 @@
 // the parity of j & z splits into a part of the thread and a part of k that the whole grid shares.
 // Bound by shared-memory reads (one amplitude pair per mask) and FP32 / FP64 issue, no longer by HBM:
 // a Heisenberg chain of 26 qubits (25 bond masks, 75 terms, and the field) took 14.6 ms with one pass
-// per mask and takes 1.27 ms (24 qubits in complex128: 2.03).  Three CTAs fit an SM (64 KiB of tile each,
+// per mask and takes 1.33 ms (24 qubits in complex128: 2.03).  Three CTAs fit an SM (64 KiB of tile each,
 // terms and offsets behind it as many as there are: two CTAs 1.76 ms, three 1.37); terms whose sign is the
 // same for all pairs of a thread, most of a chain's, share one sum (1.37 -> 1.27 ms, complex128 2.99 -> 2.03).
 #include <cuda_runtime.h>
@@ -146,6 +146,10 @@ __global__ void __launch_bounds__(kThreads, 3) pauli_tile_kernel(const typename 
             if (q.tmid < q.t1) {
                 values(true);
                 terms(q.tmid, q.t1);
+            }
+            if (sizeof(R) == 4 && (g & 3) == 3) {  // FP32 sums stay as short as with one pass per mask (1.27 -> 1.33 ms)
+                acc += (double)facc;
+                facc = 0;
             }
         }
         acc += (double)facc;
