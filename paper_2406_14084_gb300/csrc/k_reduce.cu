@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kRedThreads) expect_wht_kernel(const typename 
 // shared memory where they share their bins, and the rest with one FP64 atomic per CTA or warp and bin
 // (none where a bin belongs to one warp).  Bound by HBM (complex64) or the FP64 pipe (complex128, two
 // FMAs per amplitude).  The kernels before added each amplitude into a shared-memory histogram with an
-// FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.22) or kept every bin in registers with one
+// FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.21) or kept every bin in registers with one
 // select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.39).
 struct ProbsPlan {
     uint64_t hs, hn;      // selected / other bits above the low ones
@@ -365,6 +365,31 @@ __device__ __forceinline__ uint64_t deposit(uint64_t i, uint64_t mask)
         if (i & 1) r |= mask & (~mask + 1);
     return r;
 }
+
+// Sum of squares in float-float form, eight amplitudes at a time: squares exact (two-product), sums by two-sum,
+// about 48 bits.  Bins of 2^14 to 2^27 amplitudes are within 9e-15 of their exact sums (histograms of FP64
+// atomics: 1.7e-14; FP32 sums of 32 amplitudes, which this replaces: 6e-8, 0.22 ms where this takes 0.21).  Exact
+// products need 2^-50 <= |x| (or 0), sums |x| < 2^60; amplitudes outside take FP64, which has 2 FMAs per SM and
+// clock for what these instructions do at 128.
+struct SquareSum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x, float y)
+    {
+        const float px = __fmul_rn(x, x), py = __fmul_rn(y, y);
+        const float ex = __fmaf_rn(x, x, -px), ey = __fmaf_rn(y, y, -py);
+        const float s = __fadd_rn(px, py), b = __fsub_rn(s, px);
+        const float e = __fadd_rn(__fsub_rn(px, __fsub_rn(s, b)), __fsub_rn(py, b));
+        const float t = __fadd_rn(h, s), c = __fsub_rn(t, h);
+        const float g = __fadd_rn(__fsub_rn(h, __fsub_rn(t, c)), __fsub_rn(s, c));
+        h = t;
+        l = __fadd_rn(l, __fadd_rn(__fadd_rn(ex, ey), __fadd_rn(e, g)));
+    }
+    __device__ __forceinline__ void flush(double &acc)
+    {
+        acc += (double)h + (double)l;
+        h = l = 0.f;
+    }
+};
 
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>::T *__restrict__ a,
@@ -395,16 +420,13 @@ __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>
         const bool has = unit < units;
         const uint64_t fixed = deposit(unit >> p.logc, p.hs) | deposit(unit & ((1ull << p.logc) - 1), chunk) | mine;
         double acc[1 << VL] = {};
-        R f[1 << VL] = {};
-        auto add = [&](const auto &v) {  // one load's amplitudes
+        SquareSum f[1 << VL];  // complex64
+        auto add64 = [&](const auto &v) {  // one load's amplitudes
+            acc[0] = fma((double)v.x, (double)v.x, acc[0]);
+            acc[0] = fma((double)v.y, (double)v.y, acc[0]);
             if constexpr (VL == 1) {
-                f[0] = fmaf(v.x, v.x, f[0]);
-                f[0] = fmaf(v.y, v.y, f[0]);
-                f[VL] = fmaf(v.z, v.z, f[VL]);
-                f[VL] = fmaf(v.w, v.w, f[VL]);
-            } else {
-                acc[0] = fma(v.x, v.x, acc[0]);
-                acc[0] = fma(v.y, v.y, acc[0]);
+                acc[VL] = fma((double)v.z, (double)v.z, acc[VL]);
+                acc[VL] = fma((double)v.w, (double)v.w, acc[VL]);
             }
         };
         using V = std::conditional_t<VL == 1, float4, double2>;
@@ -415,22 +437,49 @@ __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>
                     V v[U];
 #pragma unroll
                     for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const V *>(a + (fixed | x | off[u])));
+                    if constexpr (VL == 1) {
+                        uint32_t least = ~0u;
+                        float most = 0.f;
 #pragma unroll
-                    for (int u = 0; u < U; ++u) add(v[u]);
-                    if (VL == 1 && (it & 3) == 3) {  // FP32 partial sums of at most 32 amplitudes
-                        acc[0] += (double)f[0];
-                        acc[VL] += (double)f[VL];
-                        f[0] = f[VL] = R(0);
+                        for (int u = 0; u < U; ++u) {
+                            const float w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                least = min(least, 2u * __float_as_uint(w[k]) - 1u);  // (zeros are the largest)
+                                most = fmaxf(most, fabsf(w[k]));
+                            }
+                        }
+                        // (up to five qubits the sums have always been FP32: no look for small ones)
+                        if ((p.nq <= 5 || least >= 2u * __float_as_uint(0x1p-50f) - 1u) && most < 0x1p60f) {
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                f[0].add(v[u].x, v[u].y);
+                                f[VL].add(v[u].z, v[u].w);
+                            }
+                        } else {
+#pragma unroll 1
+                            for (int u = 0; u < U; ++u) {
+                                V t = v[0];
+#pragma unroll
+                                for (int k = 1; k < U; ++k) t = u == k ? v[k] : t;
+                                add64(t);
+                            }
+                        }
+                        f[0].flush(acc[0]);
+                        f[VL].flush(acc[VL]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < U; ++u) add64(v[u]);
                     }
                     x = ((x | ~rest) + 1) & rest;  // the next subset of rest
                 }
             } else {  // fewer than eight loads in all
                 for (uint32_t u = 0; u < (1u << nu); ++u)
-                    add(__ldcs(reinterpret_cast<const V *>(a + (fixed | deposit(u, inner)))));
+                    add64(__ldcs(reinterpret_cast<const V *>(a + (fixed | deposit(u, inner)))));
             }
         }
 #pragma unroll
-        for (int k = 0; k < (1 << VL); ++k) acc[k] += (double)f[k];
+        for (int k = 0; k < (1 << VL); ++k) f[k].flush(acc[k]);
         // lanes (and halves) of one bin; selected low bits keep them apart
         uint32_t keep = 0;
         for (int j = 0; j < p.nq; ++j)
