@@ -164,9 +164,11 @@ struct Builder {
         }
         push(std::move(t));
     }
+    // Only phases of modulus 1: on a flipped bit the record needs 1 / p, which a projector (p = 0) or a
+    // small p does not have; such a diagonal stays a record of its own or goes into a table.
     bool join_sep(LeanItem &t, const LeanItem &ph) const
     {
-        if (ph.lcm || ph.ocm || __builtin_popcount(ph.rd) > 1) return false;
+        if (ph.lcm || ph.ocm || __builtin_popcount(ph.rd) > 1 || !(std::abs(std::norm(ph.p) - 1.0) <= 1e-12)) return false;
         std::vector<cd> &tab = t.sep[0].tab;
         const bool e0 = ph.m32 & 1u;
         for (size_t h = 0; h < tab.size(); h += RB + 1) {

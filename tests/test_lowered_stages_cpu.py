@@ -1,0 +1,76 @@
+"""Records of the in-place stage engine against the sub-ops that they stand for, executed on the host
+(lowered_stages.cpp) with the records' numbers rounded as the device holds them: conditional phases on
+every pair of qubits, so that separable records appear, with X gates and wide rotations that hold register
+bits flipped, and diagonals and matrices that are not unitary.
+
+Tolerance, relative to the largest amplitude of a group: a record rounds its numbers once, at most a few
+hundred records per stage, errors adding at random: 1e-5 (FP32), 1e-12 (double-float, 48 bits), 1e-13
+(FP64)."""
+import ctypes
+import math
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2406_14084_gb300 import qs
+from paper_2406_14084_gb300 import workloads as W
+from paper_2406_14084_gb300.workloads import Gate
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+FORMS = {"c64": (dict(dtype=qs.QS_C64), 1e-5), "c128": (dict(dtype=qs.QS_C128), 1e-13),
+         "df": (dict(dtype=qs.QS_C128, arith=qs.QS_ARITH_DF), 1e-12)}
+
+
+@pytest.fixture(scope="module")
+def compare(tmp_path_factory):
+    qs.lib()
+    so, lib = qs.library_path(), str(tmp_path_factory.mktemp("lowered") / "lowered_stages.so")
+    pkg = os.path.dirname(os.path.abspath(qs.__file__))
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(pkg, "..", "include"), "-I",
+                    os.path.join(pkg, "csrc"), os.path.join(HERE, "lowered_stages.cpp"), so, "-o", lib,
+                    "-Wl,-rpath," + os.path.dirname(so)], check=True)
+    fn = ctypes.CDLL(lib).lowered_difference
+    fn.restype = ctypes.c_double
+
+    def run(gates, n, **kw):
+        """Largest difference and (stages, lowered stages, separable records, records)."""
+        arr, keep = qs.marshal_gates(gates)
+        opts, count = qs.options(**kw), (ctypes.c_int64 * 4)()
+        worst = fn(arr, ctypes.c_size_t(len(gates)), n, ctypes.byref(opts), count)
+        del keep
+        assert worst >= 0.0
+        return worst, tuple(count)
+
+    return run
+
+
+def pairs(n, seed, diagonals):
+    """Controlled phases on every pair between X gates, rotations and the given one-qubit diagonals."""
+    rng = W.SplitMix64(seed)
+    out = [Gate("H", (q,)) for q in range(n)] + [Gate("X", (q,)) for q in range(n) if rng.below(2)]
+    for a in range(n):
+        out += [Gate("CP", (a, b), (), (rng.angle(),)) for b in range(a + 1, n)]
+        if rng.below(3) == 0:
+            out.append(Gate("X", (a,)))
+        if rng.below(4) == 0:
+            out.append(Gate("RY", (rng.below(n),), (), (math.pi - 0.01 * rng.uniform(),)))
+        if diagonals and rng.below(3) == 0:
+            out.append(Gate("DIAG", (rng.below(n),), (), (), np.array(diagonals[rng.below(len(diagonals))], dtype=complex)))
+    return out
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("fuse", [0, 2])
+@pytest.mark.parametrize("diagonals", [None, ((1, 0),), ((0, 1), (1, 0)), ((1, 1e-3), (0.5, 1)), ((0, 0),)],
+                         ids=["unitary", "zero", "zeros", "moduli", "null"])
+def test_separable_records_with_any_diagonal(compare, diagonals, fuse, form):
+    opts, tol = FORMS[form]
+    separable = 0
+    for seed in range(24):
+        n = (10, 13, 16)[seed % 3]
+        worst, count = compare(pairs(n, seed, diagonals), n, fuse_width=fuse, slab_bits=(0, 9)[seed % 2], **opts)
+        assert worst <= tol, (seed, worst)
+        separable += count[2]
+    assert separable or form == "c128"  # FP64 tables take more conditions and mostly stay cheaper
