@@ -19,11 +19,13 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <type_traits>
 #include <unordered_map>
 #include <vector>
 
 #include "qs_internal.h"
+#include "staging.h"
 
 namespace qs {
 namespace {
@@ -679,8 +681,7 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
     auto aligned = [](void *p) { return (reinterpret_cast<uintptr_t>(p) + 255) & ~uintptr_t(255); };
     WhtTerms *dpt = reinterpret_cast<WhtTerms *>(aligned(dgrp + 1));
     void *dtile = reinterpret_cast<void *>(aligned(dpt + 1));
-    // Terms by X mask, in order of first appearance, at most kMaxTermsPerGroup each.  (Host staging: a
-    // copy from pageable memory has left it when the call returns.)
+    // Terms by X mask, in order of first appearance, at most kMaxTermsPerGroup each.
     std::vector<PauliXGroup> groups;
     {
         std::unordered_map<uint64_t, int> open;  // X mask -> the group that still takes terms
@@ -695,6 +696,9 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
             groups[it->second].c.push_back(coeff[i]);
         }
     }
+    // One host image per launch, 32 launches between waits (at most 360 KiB).
+    auto wait = [st] { cudaStreamSynchronize(st); };
+    StagingRing<decltype(wait)> staging(std::max({pauli_tile_bytes(), sizeof(TermGroup), sizeof(WhtTerms)}), 32, wait);
     if (cudaMemsetAsync(res, 0, 2 * sizeof(double), st) != cudaSuccess) return cuda_fail("expect memset", err, errlen);
     // X masks with few terms share reads of the state (k_pauli.cu).  A term costs a tile pass about 2
     // operations per pair of amplitudes, so up to 8 terms per mask are well below a pass of their own.
@@ -702,29 +706,27 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
     std::vector<char> done(groups.size(), 0);
     for (size_t g = 0; g < groups.size(); ++g)
         if (groups[g].xm != 0 && groups[g].zm.size() <= 8) tiles.push_back(int(g));
-    std::vector<char> htile(pauli_tile_bytes());
     while (!tiles.empty()) {
         const std::vector<int> before = tiles;
-        const int b = pauli_tile_plan(c, groups, tiles, htile.data());
+        void *const htile = staging.next();
+        const int b = pauli_tile_plan(c, groups, tiles, htile);
         if (b == 0) {
             tiles.erase(tiles.begin());  // more X bits than a tile holds: a pass of its own below
             continue;
         }
         for (int g : before) done[g] = 1;
         for (int g : tiles) done[g] = 0;
-        if (cudaMemcpyAsync(dtile, htile.data(), htile.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        if (cudaMemcpyAsync(dtile, htile, pauli_tile_bytes(), cudaMemcpyHostToDevice, st) != cudaSuccess)
             return cuda_fail("expect upload", err, errlen);
-        const int nblk = launch_pauli_tile(c, dtile, htile.data(), b, part, kRedBlocksMax);
+        const int nblk = launch_pauli_tile(c, dtile, htile, b, part, kRedBlocksMax);
         finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
         int rc = cuda_fail("expect launch", err, errlen);
         if (rc) return rc;
     }
-    std::vector<TermGroup> hgv(1);
-    TermGroup &hg = hgv[0];
-    std::vector<WhtTerms> hw(1);
     for (size_t gi = 0; gi < groups.size(); ++gi) {
         if (done[gi]) continue;
         const PauliXGroup &G = groups[gi];
+        TermGroup &hg = *new (staging.next()) TermGroup;
         hg.xm = G.xm;
         hg.nterms = int(G.zm.size());
         for (int j = 0; j < hg.nterms; ++j) {
@@ -737,7 +739,7 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
         int nblk = blocks;
         if (hg.nterms >= 4 && c.n >= 16) {
             // Walsh-Hadamard tiles; coefficients folded on the host in FP64
-            WhtTerms &w = hw[0];
+            WhtTerms &w = *new (staging.next()) WhtTerms;
             w.xm = hg.xm;
             w.nterms = hg.nterms;
             w.pair = (hg.xm >> kWhtTileLog) != 0;
@@ -778,6 +780,7 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
     if (cudaMemcpyAsync(h_out, res, 2 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return cuda_fail("expect readback", err, errlen);
+    staging.idle();
     return QS_OK;
 }
 
