@@ -78,6 +78,7 @@ struct DevPlanBuf {
     std::vector<Lean> lean;
     int device = -1;
     bool borrowed = false;    // base is a state's plan_ws, not the plan's own
+    std::unique_ptr<unsigned char[]> host;  // borrowed: source of the copy under way to base
 };
 
 constexpr size_t kPlanWsMax = size_t(8) << 20;  // larger plans get their own allocation
@@ -192,7 +193,8 @@ qs_status ensure_scratch(qs_state *s, size_t bytes)
     return QS_OK;
 }
 
-// borrow: put the plan into this state's plan_ws (the caller synchronises before it returns)
+// borrow: put the plan into this state's plan_ws.  The copy is asynchronous and may read its source until the
+// stream has been waited for, so the plan keeps it and the caller waits before it drops the plan (Drain).
 qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
 {
     DevPlanBuf &d = pl->dev[dt];
@@ -244,7 +246,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     const size_t o_coef = section((nc + 2) * amp_bytes(dt));
     const size_t o_cdf = section(want_df ? (nc + 2) * 16 : 0);
     const size_t o_words = section(img.words.size()), o_pool = section(img.pool.size());
-    const std::unique_ptr<unsigned char[]> h(new unsigned char[total]);  // (padding stays unset)
+    std::unique_ptr<unsigned char[]> h(new unsigned char[total]);  // (padding stays unset)
     auto fill = [&](size_t off, const void *src, size_t bytes) {
         if (bytes) std::memcpy(h.get() + off, src, bytes);
     };
@@ -310,6 +312,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
         base = borrow->plan_ws;
         st = cuda_status(cudaMemcpyAsync(base, h.get(), total, cudaMemcpyHostToDevice, borrow->stream), "plan upload");
         if (st) return st;
+        d.host = std::move(h);
     } else {
         st = cuda_status(cudaMalloc(&base, total), "plan upload allocation");
         if (st) return st;
@@ -366,6 +369,12 @@ struct StepTimer {
         cudaEventElapsedTime(&ms, ev[i], ev[j]);
         return ms;
     }
+};
+
+// Waits for a stream on every way out; declared after the plan that the stream still reads.
+struct Drain {
+    cudaStream_t stream;
+    ~Drain() { cudaStreamSynchronize(stream); }
 };
 
 // transient: the plan lives within the caller's call (see upload)
@@ -443,9 +452,8 @@ qs_status canonicalize_state(qs_state *s)
     pl->p.n = s->n;
     pl->p.dt = s->dt;
     plan_canonicalize(s->n, s->dt, s->phys_of, pl->p);
+    const Drain drain{s->stream};
     qs_status st = run_plan(s, pl.get(), nullptr, true);
-    // wait: the plan's device memory is reused or freed after this call
-    cudaStreamSynchronize(s->stream);
     if (st) return st;
     for (int q = 0; q < s->n; ++q) s->phys_of[q] = q;
     return QS_OK;
@@ -1040,9 +1048,8 @@ qs_status qs_apply_circuit(qs_state *s, const qs_gate *g, size_t ng, const qs_op
     qs_status st = qs_fuse(g, ng, s->n, &opt, &p);
     if (st) return st;
     std::unique_ptr<qs_plan> own(p);
-    st = apply_plan(s, p, true);
-    cudaStreamSynchronize(s->stream);
-    return st;
+    const Drain drain{s->stream};
+    return apply_plan(s, p, true);
     QS_GUARD_END
 }
 
@@ -1057,8 +1064,8 @@ qs_status qs_remap(qs_state *s, int k, const int *A, const int *B)
     std::string err;
     int rc = plan_remap(s->n, s->dt, a, b, pl->p, err);
     if (rc) return fail((qs_status)rc, err);
+    const Drain drain{s->stream};
     qs_status st = run_plan(s, pl.get(), nullptr, true);
-    cudaStreamSynchronize(s->stream);
     if (st) return st;
     std::vector<int> logi(s->n);
     for (int q = 0; q < s->n; ++q) logi[s->phys_of[q]] = q;
