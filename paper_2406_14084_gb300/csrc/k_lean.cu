@@ -5,7 +5,7 @@
 // an SM and one computes while the other loads or stores.  Measured with the stage engine, whole
 // circuits: layered-28 complex64 (20 layers, 14 passes) 89.5 -> 41 ms, complete-graph QAOA-23
 // complex64 2.94 -> 0.82 ms, QFT-28 complex128 110 -> 83 ms (FP64 pipe 90 % busy), layered-25
-// complex128 104 -> 96 ms, layered-26 in double-float form 60.9 -> 36.8 ms.
+// complex128 104 -> 96 ms, layered-26 in double-float form 60.9 -> 38.1 ms.
 #include <cuda_runtime.h>
 
 #include <cstdio>

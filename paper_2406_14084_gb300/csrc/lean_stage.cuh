@@ -13,7 +13,7 @@
 //                bits 413 (FMA pipe, about 80 % busy), on one bit 114, table 292-400 (L1 to
 //                registers: 256 B per thread), X 190
 //   complex128   2x2 matrix 1980, table 4330, half table 2170: the FP64 pipe, 2.0 FMA per SM and clock
-//   double-float shears on one bit 530 (FMA pipe), table 1030-1130
+//   double-float 2x2 matrix 550 (FMA pipe), table 1030-1130
 #pragma once
 
 #include "slab_common.cuh"
@@ -448,16 +448,29 @@ __device__ __forceinline__ void df_prod(const df_factor &a, const dfp &b, unsign
     g = fma2(a.nh, b.l, g);
     g = fma2(a.nl, b.h, g);
 }
-__device__ __forceinline__ dfp df_fma(const df_factor &a, const dfp &b, const dfp &c)
+// a b + c as an unnormalised sum h + l, and in normal form
+__device__ __forceinline__ dfp df_fma_sum(const df_factor &a, const dfp &b, const dfp &c)
 {
     unsigned long long p, g;
     df_prod(a, b, p, g);
     const unsigned long long s = add2(p, c.h), bb = sub2(s, p);
-    const unsigned long long t = add2(add2(sub2(p, sub2(s, bb)), sub2(c.h, bb)), sub2(c.l, g));
+    return dfp{s, add2(add2(sub2(p, sub2(s, bb)), sub2(c.h, bb)), sub2(c.l, g))};
+}
+__device__ __forceinline__ dfp df_normal(const dfp &u)
+{
     dfp r;
-    r.h = add2(s, t);
-    r.l = sub2(t, sub2(r.h, s));
+    r.h = add2(u.h, u.l);
+    r.l = sub2(u.l, sub2(r.h, u.h));
     return r;
+}
+__device__ __forceinline__ dfp df_fma(const df_factor &a, const dfp &b, const dfp &c) { return df_normal(df_fma_sum(a, b, c)); }
+// a b - c, the same steps on -c
+__device__ __forceinline__ dfp df_fms(const df_factor &a, const dfp &b, const dfp &c)
+{
+    unsigned long long p, g;
+    df_prod(a, b, p, g);
+    const unsigned long long s = sub2(p, c.h), bb = sub2(s, p);
+    return df_normal(dfp{s, sub2(sub2(sub2(p, sub2(s, bb)), add2(c.h, bb)), add2(c.l, g))});
 }
 __device__ __forceinline__ dfp df_mul(const df_factor &a, const dfp &b)
 {
@@ -492,8 +505,10 @@ template <int RB> struct LeanRegs<dfp, RB> {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             if (e & (1 << J)) continue;
-            v[e | (1 << J)] = df_fma(y, v[e], v[e | (1 << J)]);
-            v[e] = df_fma(x, v[e | (1 << J)], v[e]);
+            // (normalised last: the sum is what waits for the other result, no copy of an input)
+            const dfp b = v[e | (1 << J)], u = df_fma_sum(x, b, v[e]);
+            v[e | (1 << J)] = NEG ? df_fms(y, v[e], b) : df_fma(y, v[e], b);
+            v[e] = df_normal(u);
         }
     }
     static __device__ __forceinline__ float4 factor(ulonglong2 w)

@@ -20,7 +20,7 @@ struct LeanItem {
     LeanOp op = L_ROTA;
     int j = 0, ctrl = -1;           // L_CX: target and control register bit (-1: none)
     uint32_t mask = 0;              // L_ROTA: register bits with a shear pair
-    // L_ROTA, per register bit: v1 += y v0, then v0 += x v1; FP64 (from both old values): v0 + x v1,
+    // L_ROTA, per register bit: v1 += y v0, then v0 += x v1; complex128 (from both old values): v0 + x v1,
     // y v0 +- v1 (minus where neg has the bit)
     double y[6] = {}, x[6] = {};
     uint32_t neg = 0;

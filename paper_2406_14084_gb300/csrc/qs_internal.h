@@ -122,10 +122,10 @@ static_assert(sizeof(DevStage) % 8 == 0, "DevStage is read with 8-byte loads");
 // word {u32 slab-local bits, -, u64 outside bits} that must all be 1.
 enum LeanOp : uint8_t {
     L_ROT0 = 0,   // L_ROT0 + j: (y, x) of register bit j, complex64 in the word's upper half, else in
-                  // a word of its own: v1 += y v0; v0 += x v1.  FP64: v0 + x v1, y v0 + v1 (old
+                  // a word of its own: v1 += y v0; v0 += x v1.  complex128: v0 + x v1, y v0 + v1 (old
                   // values)
     L_ROT1, L_ROT2, L_ROT3, L_ROT4,
-    L_ROTM0,      // FP64: v0 + x v1, y v0 - v1
+    L_ROTM0,      // complex128: v0 + x v1, y v0 - v1
     L_ROTM1, L_ROTM2, L_ROTM3,
     L_ROTA,       // complex64: (y, x) of every register bit, from the upper half on, two per word
     L_CONST,      // u32 at byte 8 = pattern that holds the factors other than 1; all factors follow

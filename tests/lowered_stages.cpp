@@ -115,7 +115,7 @@ extern "C" double lowered_difference(const qs_gate *g, size_t ng, int n, const q
                         for (uint32_t e = 0; e < E; ++e) {
                             if (!(it.mask >> j & 1) || (e >> j & 1)) continue;
                             cd &a = u[e], &b = u[e | 1u << j];
-                            if (dt == QS_C128 && !df) {
+                            if (dt == QS_C128) {
                                 const cd a0 = a;
                                 a = a0 + D(it.x[j]) * b;
                                 b = D(it.y[j]) * a0 + ((it.neg >> j & 1) ? -b : b);
