@@ -451,8 +451,7 @@ __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>
                                 most = fmaxf(most, fabsf(w[k]));
                             }
                         }
-                        // (up to five qubits the sums have always been FP32: no look for small ones)
-                        if ((p.nq <= 5 || least >= 2u * __float_as_uint(0x1p-50f) - 1u) && most < 0x1p60f) {
+                        if (least >= 2u * __float_as_uint(0x1p-50f) - 1u && most < 0x1p60f) {
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
                                 f[0].add(v[u].x, v[u].y);
