@@ -348,19 +348,26 @@ __global__ void __launch_bounds__(kRedThreads) expect_wht_kernel(const typename 
 // above, which the warp runs over.  Each lane so adds into one or two sums that belong to one bin
 // whatever nq is; at the end lanes of the same bin are added with shuffles, the eight warps of a CTA in
 // shared memory where they share their bins, and the rest with one FP64 atomic per CTA or warp and bin
-// (none where a bin belongs to one warp).  Bound by HBM (complex64) or the FP64 pipe (complex128, two
-// FMAs per amplitude).  The kernels before added each amplitude into a shared-memory histogram with an
-// FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.21) or kept every bin in registers with one
-// select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.39).
+// (none where a bin belongs to one warp or CTA).  Bound by HBM (complex64) or the FP64 pipe (complex128,
+// two FMAs per amplitude).  The kernels before added each amplitude into a shared-memory histogram with an
+// FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.19) or kept every bin in registers with one
+// select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.39).  Masks and offsets
+// come from the host: small states wait for the chain of dependent instructions, not for memory.
 struct ProbsPlan {
-    uint64_t hs, hn;      // selected / other bits above the low ones
-    int ns, nn, logc;     // their counts; log2 of the warps that share one setting of hs
-    int low, nq;          // number of low bits
+    uint64_t hs;          // selected bits above the low ones
+    uint64_t chunk, rest; // other bits above: told apart by warps that share hs; run over, eight loads a step
+    uint64_t off[8];      // offsets of the loads of one step
+    int ns, nn, logc;     // number of selected / other bits above; log2 of the warps that share one setting of hs
+    int gb;               // log2 of the settings of hs in one step (probs_bins_kernel)
+    int low, nq;          // number of low bits; of selected ones
+    uint32_t keep;        // selected low bits
+    uint32_t mhalf;       // index bit of the selection's index bit 0 (complex64), 0 if it is not selected
     uint8_t pos[32];
+    uint8_t hpos[24], hidx[24];  // selected bits above: position, and place in the bin's number
 };
 
 // the i-th (bit-wise) subset of mask
-__device__ __forceinline__ uint64_t deposit(uint64_t i, uint64_t mask)
+__host__ __device__ inline uint64_t deposit(uint64_t i, uint64_t mask)
 {
     uint64_t r = 0;
     for (; i != 0; i >>= 1, mask &= mask - 1)
@@ -370,7 +377,7 @@ __device__ __forceinline__ uint64_t deposit(uint64_t i, uint64_t mask)
 
 // Sum of squares in float-float form, eight amplitudes at a time: squares exact (two-product), sums by two-sum,
 // about 48 bits.  Bins of 2^14 to 2^27 amplitudes are within 9e-15 of their exact sums (histograms of FP64
-// atomics: 1.7e-14; FP32 sums of 32 amplitudes, which this replaces: 6e-8, 0.22 ms where this takes 0.21).  Exact
+// atomics: 1.7e-14; FP32 sums of 32 amplitudes: 6e-8, and no faster).  Exact
 // products need 2^-50 <= |x| (or 0), sums |x| < 2^60; amplitudes outside take FP64, which has 2 FMAs per SM and
 // clock for what these instructions do at 128.
 struct SquareSum {
@@ -381,142 +388,241 @@ struct SquareSum {
         const float ex = __fmaf_rn(x, x, -px), ey = __fmaf_rn(y, y, -py);
         const float s = __fadd_rn(px, py), b = __fsub_rn(s, px);
         const float e = __fadd_rn(__fsub_rn(px, __fsub_rn(s, b)), __fsub_rn(py, b));
+        join(s, __fadd_rn(__fadd_rn(ex, ey), e));
+    }
+    // adds another sum
+    __device__ __forceinline__ void join(float s, float r)
+    {
         const float t = __fadd_rn(h, s), c = __fsub_rn(t, h);
         const float g = __fadd_rn(__fsub_rn(h, __fsub_rn(t, c)), __fsub_rn(s, c));
         h = t;
-        l = __fadd_rn(l, __fadd_rn(__fadd_rn(ex, ey), __fadd_rn(e, g)));
+        l = __fadd_rn(l, __fadd_rn(r, g));
     }
+    __device__ __forceinline__ void join_lane(int mask)
+    {
+        join(__shfl_xor_sync(0xffffffffu, h, mask), __shfl_xor_sync(0xffffffffu, l, mask));
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
     __device__ __forceinline__ void flush(double &acc)
     {
-        acc += (double)h + (double)l;
+        acc += value();
         h = l = 0.f;
     }
 };
+struct Square64 {  // the same in FP64
+    double s = 0.0;
+    template <typename F> __device__ __forceinline__ void add(F x, F y)
+    {
+        s = fma((double)x, (double)x, s);
+        s = fma((double)y, (double)y, s);
+    }
+    __device__ __forceinline__ void join_lane(int mask) { s += __shfl_xor_sync(0xffffffffu, s, mask); }
+    __device__ __forceinline__ double value() const { return s; }
+};
 
+template <typename R> struct ProbsLoad;
+template <> struct ProbsLoad<float> {
+    using V = float4;
+    static constexpr int VL = 1;  // low bit inside a 16-byte load
+    // amplitudes whose squares and sums float-float numbers hold
+    template <int U> static __device__ __forceinline__ bool fits(const V (&v)[U])
+    {
+        uint32_t least = ~0u;
+        float most = 0.f;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                least = min(least, 2u * __float_as_uint(w[k]) - 1u);  // (zeros are the largest)
+                most = fmaxf(most, fabsf(w[k]));
+            }
+        }
+        return least >= 2u * __float_as_uint(0x1p-50f) - 1u && most < 0x1p60f;
+    }
+};
+template <> struct ProbsLoad<double> {
+    using V = double2;
+    static constexpr int VL = 0;
+};
+
+// lanes of one bin (selected low bits keep them apart)
+template <int VL, typename A> __device__ __forceinline__ void join_lanes(A &a, uint32_t keep)
+{
+#pragma unroll
+    for (int l = 0; l < 5; ++l)
+        if (!(keep >> (l + VL) & 1u)) a.join_lane(1 << l);
+}
+
+// Eight loads a step, and at least one step, per warp and setting of the selected bits above.
 template <typename R>
 __global__ void __launch_bounds__(kRedThreads) probs_kernel(const typename Cx<R>::T *__restrict__ a,
                                                             const __grid_constant__ ProbsPlan p, double *__restrict__ hist)
 {
-    using T = typename Cx<R>::T;
-    constexpr int VL = sizeof(T) == 8 ? 1 : 0;  // low bit inside a 16-byte load
-    constexpr int U = 8;                        // loads in flight per lane
-    __shared__ double sh[kRedThreads / 32][32][1 << VL];
+    using V = typename ProbsLoad<R>::V;
+    constexpr int VL = ProbsLoad<R>::VL, U = 8, H = 1 << VL, W = kRedThreads / 32;
+    static_assert(W == 8, "eight threads add a bin's eight warps");
+    __shared__ double sh[32 * H][W + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t units = 1ull << (p.ns + p.logc);
     const uint64_t mine = uint64_t(lane) << VL;
-    const bool live = (mine >> p.low) == 0;  // states smaller than one load per lane
-    const int nrun = p.nn - p.logc;          // bits of hn that one warp runs over: the low nrun ones
-    const uint64_t chunk = nrun >= 64 ? 0 : deposit(~0ull << nrun & ((1ull << p.nn) - 1), p.hn);  // the others
-    const uint64_t run = p.hn & ~chunk;
-    uint64_t off[U], rest = run;  // off: the loads in flight
-    int nu = 0;  // the lowest bits of run, up to three, index the loads in flight
-    for (; nu < 3 && rest != 0; ++nu) rest &= rest - 1;
-    const uint64_t inner = run & ~rest;
-#pragma unroll
-    for (int u = 0; u < U; ++u) off[u] = deposit(uint64_t(u) & ((1u << nu) - 1), inner);
-    const uint64_t iters = 1ull << (nrun - nu);
+    const uint64_t iters = 1ull << (p.nn - p.logc - 3);
     const bool joint = p.logc >= 3;  // the CTA's warps share hs
-    for (uint64_t u0 = uint64_t(blockIdx.x) * (kRedThreads / 32); u0 < units;
-         u0 += uint64_t(gridDim.x) * (kRedThreads / 32)) {
+    for (uint64_t u0 = uint64_t(blockIdx.x) * W; u0 < units; u0 += uint64_t(gridDim.x) * W) {
         const uint64_t unit = u0 + warp;
         const bool has = unit < units;
-        const uint64_t fixed = deposit(unit >> p.logc, p.hs) | deposit(unit & ((1ull << p.logc) - 1), chunk) | mine;
-        double acc[1 << VL] = {};
-        SquareSum f[1 << VL];  // complex64
-        auto add64 = [&](const auto &v) {  // one load's amplitudes
-            acc[0] = fma((double)v.x, (double)v.x, acc[0]);
-            acc[0] = fma((double)v.y, (double)v.y, acc[0]);
-            if constexpr (VL == 1) {
-                acc[VL] = fma((double)v.z, (double)v.z, acc[VL]);
-                acc[VL] = fma((double)v.w, (double)v.w, acc[VL]);
-            }
-        };
-        using V = std::conditional_t<VL == 1, float4, double2>;
-        if (has && live) {
-            if (nu == 3) {
-                uint64_t x = 0;
-                for (uint64_t it = 0; it < iters; ++it) {
-                    V v[U];
+        const uint64_t sel = deposit(unit >> p.logc, p.hs);
+        const auto *at = a + (sel | deposit(unit & ((1ull << p.logc) - 1), p.chunk) | mine);
+        Square64 acc[H];
+        if (has) {
+            uint64_t x = 0;
+            for (uint64_t it = 0; it < iters; ++it) {
+                V v[U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const V *>(a + (fixed | x | off[u])));
-                    if constexpr (VL == 1) {
-                        uint32_t least = ~0u;
-                        float most = 0.f;
+                for (int u = 0; u < U; ++u) v[u] = __ldcs(reinterpret_cast<const V *>(at + (x | p.off[u])));
+                if constexpr (VL == 1) {
+                    if (ProbsLoad<R>::fits(v)) {
+                        SquareSum f[H];
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
-                            const float w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                least = min(least, 2u * __float_as_uint(w[k]) - 1u);  // (zeros are the largest)
-                                most = fmaxf(most, fabsf(w[k]));
-                            }
+                            f[0].add(v[u].x, v[u].y);
+                            f[VL].add(v[u].z, v[u].w);
                         }
-                        if (least >= 2u * __float_as_uint(0x1p-50f) - 1u && most < 0x1p60f) {
-#pragma unroll
-                            for (int u = 0; u < U; ++u) {
-                                f[0].add(v[u].x, v[u].y);
-                                f[VL].add(v[u].z, v[u].w);
-                            }
-                        } else {
-#pragma unroll 1
-                            for (int u = 0; u < U; ++u) {
-                                V t = v[0];
-#pragma unroll
-                                for (int k = 1; k < U; ++k) t = u == k ? v[k] : t;
-                                add64(t);
-                            }
-                        }
-                        f[0].flush(acc[0]);
-                        f[VL].flush(acc[VL]);
+                        f[0].flush(acc[0].s);
+                        f[VL].flush(acc[VL].s);
                     } else {
+#pragma unroll 1
+                        for (int u = 0; u < U; ++u) {
+                            V t = v[0];
 #pragma unroll
-                        for (int u = 0; u < U; ++u) add64(v[u]);
+                            for (int k = 1; k < U; ++k) t = u == k ? v[k] : t;
+                            acc[0].add(t.x, t.y);
+                            acc[VL].add(t.z, t.w);
+                        }
                     }
-                    x = ((x | ~rest) + 1) & rest;  // the next subset of rest
+                } else {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) acc[0].add(v[u].x, v[u].y);
                 }
-            } else {  // fewer than eight loads in all
-                for (uint32_t u = 0; u < (1u << nu); ++u)
-                    add64(__ldcs(reinterpret_cast<const V *>(a + (fixed | deposit(u, inner)))));
+                x = ((x | ~p.rest) + 1) & p.rest;  // the next subset of rest
             }
         }
-#pragma unroll
-        for (int k = 0; k < (1 << VL); ++k) f[k].flush(acc[k]);
-        // lanes (and halves) of one bin; selected low bits keep them apart
-        uint32_t keep = 0;
-        for (int j = 0; j < p.nq; ++j)
-            if (p.pos[j] < p.low) keep |= 1u << p.pos[j];
-        if (VL == 1 && !(keep & 1u)) {
-            acc[0] += acc[VL];
-            acc[VL] = acc[0];
+        if (VL == 1 && !(p.keep & 1u)) {
+            acc[0].s += acc[VL].s;
+            acc[VL].s = acc[0].s;
         }
-        bool writer = true;
-        for (int l = 0; l < 5; ++l) {
-            if (keep >> (l + VL) & 1u) continue;
 #pragma unroll
-            for (int k = 0; k < (1 << VL); ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 1 << l);
-            writer = writer && !(lane >> l & 1);
-        }
+        for (int k = 0; k < H; ++k) join_lanes<VL>(acc[k], p.keep);
+        auto store = [&](uint32_t lk, double v) {  // bin of low index lk
+            const uint64_t y = sel | lk;
+            uint32_t m = 0;
+            for (int j = 0; j < p.nq; ++j) m |= uint32_t((y >> p.pos[j]) & 1) << j;
+            if (p.logc == 0 || p.logc == 3) hist[m] = v;
+            else atomicAdd(&hist[m], v);
+        };
+        // (of the lanes and halves of a bin, the one whose other low bits are 0 stores it)
         if (joint) {
 #pragma unroll
-            for (int k = 0; k < (1 << VL); ++k) sh[warp][lane][k] = acc[k];
+            for (int k = 0; k < H; ++k) sh[(lane << VL) | k][warp] = acc[k].s;
             __syncthreads();
-            if (warp == 0) {
+            // eight threads a sum; (32 H) of them, 32 at a time
+            for (uint32_t lk = threadIdx.x >> 3; lk < 32u * H; lk += kRedThreads / 8) {
+                double v = sh[lk][threadIdx.x & 7];
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                v += __shfl_xor_sync(0xffffffffu, v, 4);
+                if ((threadIdx.x & 7) == 0 && (lk & ~p.keep) == 0) store(lk, v);
+            }
+            __syncthreads();
+        } else if (has) {
 #pragma unroll
-                for (int k = 0; k < (1 << VL); ++k)
-                    for (int w = 1; w < kRedThreads / 32; ++w) acc[k] += sh[w][lane][k];
-            }
-            __syncthreads();
-            writer = writer && warp == 0;
+            for (int k = 0; k < H; ++k)
+                if (((uint32_t(mine) | k) & ~p.keep) == 0) store(uint32_t(mine) | k, acc[k].s);
         }
-        if (writer && has && live) {
-            const uint64_t x = deposit(unit >> p.logc, p.hs) | mine;
-            const int halves = VL == 1 && (keep & 1u) ? 2 : 1;
-            for (int k = 0; k < halves; ++k) {
-                uint32_t m = 0;
-                for (int j = 0; j < p.nq; ++j) m |= uint32_t(((x | uint64_t(k)) >> p.pos[j]) & 1) << j;
-                if (p.logc == 0) hist[m] = acc[k];
-                else atomicAdd(&hist[m], acc[k]);
+    }
+}
+
+// Nearly all bits above the low ones selected (NN = 0, 1 or 2 are not), and states smaller than a few loads per
+// lane: a step's eight loads belong to 2^(3-NN) settings of the selected bits.  (One setting at a time left
+// one to four loads in flight and spent a loop over the bits on each: the upper 20 of 27 qubits 1.91 -> 0.44 ms
+// in complex64, of 26 qubits in complex128 1.40 -> 0.67; atomics into device memory took 1.41 and 0.70.)  With
+// fewer settings than resident warps, each has a warp of its own.
+template <typename R, int NN>
+__global__ void __launch_bounds__(kRedThreads) probs_bins_kernel(const typename Cx<R>::T *__restrict__ a,
+                                                                 const __grid_constant__ ProbsPlan p, double *__restrict__ hist)
+{
+    using V = typename ProbsLoad<R>::V;
+    constexpr int VL = ProbsLoad<R>::VL, U = 8, H = 1 << VL, W = kRedThreads / 32, G = U >> NN;
+    const int lane = threadIdx.x & 31;
+    const int gb = p.gb;
+    const uint64_t units = 1ull << (p.ns - gb);
+    const uint64_t mine = uint64_t(lane) << VL;
+    const bool live = (mine >> p.low) == 0;  // states smaller than one load per lane
+    const bool writer = live && (uint32_t(mine) & ~(p.keep | (H - 1u))) == 0;
+    uint32_t ml = 0, mg[G];
+    for (int j = 0; j < p.nq; ++j)
+        if (p.pos[j] < p.low) ml |= uint32_t((mine >> p.pos[j]) & 1) << j;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        mg[g] = 0;
+#pragma unroll
+        for (int j = 0; j < 3 - NN; ++j)
+            if (j < gb && (g >> j & 1)) mg[g] |= 1u << p.hidx[j];
+    }
+    for (uint64_t unit = uint64_t(blockIdx.x) * W + (threadIdx.x >> 5); unit < units; unit += uint64_t(gridDim.x) * W) {
+        uint64_t x = mine;
+        uint32_t m = ml;
+        for (int j = gb; j < p.ns; ++j) {
+            const uint64_t bit = (unit >> (j - gb)) & 1;
+            x |= bit << p.hpos[j];
+            m |= uint32_t(bit) << p.hidx[j];
+        }
+        V v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v[u] = V{};
+            if (live && (u >> NN) < (1 << gb)) v[u] = __ldcs(reinterpret_cast<const V *>(a + (x | p.off[u])));
+        }
+        auto bins = [&](auto zero) {
+            using A = decltype(zero);
+            A s[G][H];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if (g && g >= (1 << gb)) continue;
+#pragma unroll
+                for (int i = 0; i < (1 << NN); ++i) {
+                    const V t = v[(g << NN) | i];
+                    s[g][0].add(t.x, t.y);
+                    if constexpr (VL == 1) {
+                        if (p.mhalf) s[g][VL].add(t.z, t.w);
+                        else s[g][0].add(t.z, t.w);
+                    }
+                }
             }
+            // lane bits outside, bins inside: each exchange of one bin hides behind those of the others
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {
+                if (p.keep >> (l + VL) & 1u) continue;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    if (g && g >= (1 << gb)) continue;
+                    s[g][0].join_lane(1 << l);
+                    if (VL == 1 && p.mhalf) s[g][VL].join_lane(1 << l);
+                }
+            }
+            if (!writer) return;
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if (g && g >= (1 << gb)) continue;
+                hist[m | mg[g]] = s[g][0].value();
+                if (VL == 1 && p.mhalf) hist[m | mg[g] | p.mhalf] = s[g][VL].value();
+            }
+        };
+        if constexpr (VL == 1) {
+            if (__all_sync(0xffffffffu, ProbsLoad<R>::fits(v))) bins(SquareSum{});
+            else bins(Square64{});
+        } else {
+            bins(Square64{});
         }
     }
 }
@@ -530,14 +636,35 @@ ProbsPlan probs_plan(int n, qs_dtype dt, const int *pos, int nq)
     for (int j = 0; j < nq; ++j) {
         p.pos[j] = uint8_t(pos[j]);
         sel |= 1ull << pos[j];
+        if (dt == QS_C64 && pos[j] == 0) p.mhalf = 1u << j;
     }
-    const uint64_t above = ((1ull << n) - 1) & ~((1ull << p.low) - 1);
+    const uint64_t lowm = (1ull << p.low) - 1, above = ((1ull << n) - 1) & ~lowm;
+    p.keep = uint32_t(sel & lowm);
     p.hs = sel & above;
-    p.hn = above & ~sel;
-    p.ns = __builtin_popcountll(p.hs);
-    p.nn = __builtin_popcountll(p.hn);
-    // 2^13 warps fill the GPU (6.7 CTAs of eight per SM); below eight loads per warp fewer share a bin
+    for (int q = 0; q < n; ++q)
+        if (p.hs >> q & 1) {
+            p.hpos[p.ns] = uint8_t(q);
+            p.hidx[p.ns++] = uint8_t(std::find(pos, pos + nq, q) - pos);
+        }
+    const uint64_t other = above & ~sel;
+    p.nn = __builtin_popcountll(other);
+    if (p.nn < 3) {  // loads of a step: the other bits, then the lowest selected ones
+        p.gb = std::max(0, std::min(3 - p.nn, p.ns - 11));  // (2^11 warps are resident at once)
+        for (uint32_t u = 0; u < 8; ++u)
+            p.off[u] = deposit(u & ((1u << p.nn) - 1), other) | deposit((u >> p.nn) & ((1u << p.gb) - 1), p.hs);
+        return p;
+    }
+    // 2^13 warps fill the GPU (6.7 CTAs of eight per SM).  One warp or one CTA per bin stores without a clear
+    // and atomics (3 and 10 qubits of 27: 0.21 -> 0.19 ms, with the masks from the host): two or four warps per
+    // bin are rounded to one of them, and small states use one CTA while it has 32 loads a warp at most (12
+    // qubits, 29 -> 22 us a call; at 14 qubits a launch less for 2 us more of it).
     p.logc = std::max(0, std::min(13 - p.ns, p.nn - 3));
+    if (p.logc > 3 && p.nn <= 8) p.logc = 3;
+    if (p.logc == 1 || p.logc == 2) p.logc = p.nn >= 6 ? 3 : 0;
+    p.chunk = deposit(((1ull << p.logc) - 1) << (p.nn - p.logc), other);
+    const uint64_t run = other & ~p.chunk, inner = deposit(7, run);
+    p.rest = run & ~inner;
+    for (uint32_t u = 0; u < 8; ++u) p.off[u] = deposit(u, inner);
     return p;
 }
 
@@ -601,13 +728,21 @@ int enqueue_probs(const LaunchCtx &c, const int *phys_q, int nq, double *hist, c
 {
     cudaStream_t st = (cudaStream_t)c.stream;
     const ProbsPlan p = probs_plan(c.n, c.dt, phys_q, nq);
-    if (p.logc > 0 && cudaMemsetAsync(hist, 0, (size_t(1) << nq) * sizeof(double), st) != cudaSuccess)
-        return cuda_fail("probs memset", err, errlen);
     reduce_blocks(1);  // reads the SM count once
-    const uint64_t need = ((1ull << (p.ns + p.logc)) + kRedThreads / 32 - 1) / (kRedThreads / 32);
-    const int blocks = int(std::min<uint64_t>(need, uint64_t(g_sms) * 8));
-    if (c.dt == QS_C64) probs_kernel<float><<<blocks, kRedThreads, 0, st>>>((const float2 *)c.amp, p, hist);
-    else probs_kernel<double><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, p, hist);
+    auto blocks = [](uint64_t warps) { return int(std::min<uint64_t>((warps + kRedThreads / 32 - 1) / (kRedThreads / 32), uint64_t(g_sms) * 8)); };
+    auto launch = [&](auto R, const auto *a) {
+        using T = decltype(R);
+        if (p.nn >= 3) return probs_kernel<T><<<blocks(1ull << (p.ns + p.logc)), kRedThreads, 0, st>>>(a, p, hist);
+        const int b = blocks(1ull << (p.ns - p.gb));
+        if (p.nn == 0) probs_bins_kernel<T, 0><<<b, kRedThreads, 0, st>>>(a, p, hist);
+        else if (p.nn == 1) probs_bins_kernel<T, 1><<<b, kRedThreads, 0, st>>>(a, p, hist);
+        else probs_bins_kernel<T, 2><<<b, kRedThreads, 0, st>>>(a, p, hist);
+    };
+    // bins that several CTAs add to start at 0
+    if (p.nn >= 3 && p.logc > 3 && cudaMemsetAsync(hist, 0, (size_t(1) << nq) * sizeof(double), st) != cudaSuccess)
+        return cuda_fail("probs memset", err, errlen);
+    if (c.dt == QS_C64) launch(float{}, (const float2 *)c.amp);
+    else launch(double{}, (const double2 *)c.amp);
     return cuda_fail("probs launch", err, errlen);
 }
 
