@@ -39,7 +39,9 @@ template <> struct LeanProgram<0> {
     __device__ __forceinline__ ulonglong2 operator()(uint32_t i) const { return __ldg(g + i); }
 };
 
-template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL>
+// SMALL: slabs with fewer groups than threads (states and slab options below the default slab), where whole warps
+// have none.  A variant of its own: the test costs full slabs 1 to 6 % in registers.
+template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL, bool SMALL>
 __global__ void __launch_bounds__(NT, PER_SM)
     lean_pass_kernel(typename Cx<R>::T *__restrict__ state, const __grid_constant__ LeanProgram<NW> prog,
                      const void *__restrict__ pool, uint64_t nslabs)
@@ -94,7 +96,8 @@ __global__ void __launch_bounds__(NT, PER_SM)
         uint32_t at = 0;
 #pragma unroll 1
         for (int o = 0; o < prog.nstages; ++o) {
-            if constexpr (DF)
+            if (SMALL && !with_groups(tid, b - RB)) {
+            } else if constexpr (DF)
                 at = run_lean_stage<dfp, RB, FULL>(reinterpret_cast<dfp *>(sm), prog, at, static_cast<const dfp *>(pool), base, tid);
             else
                 at = run_lean_stage<C, RB, FULL>(sm, prog, at, static_cast<const C *>(pool), base, tid);
@@ -116,12 +119,12 @@ __global__ void __launch_bounds__(NT, PER_SM)
     }
 }
 
-template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL>
+template <typename R, int RB, int NT, int PER_SM, bool DF, int NW, bool FULL, bool SMALL = false>
 int launch_lean_t(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h, char *err, size_t errlen)
 {
     using C = typename Cx<R>::T;
     const size_t smem = (sizeof(C) << h.b) + (sizeof(uint64_t) << h.nhi);
-    auto *const kern = lean_pass_kernel<R, RB, NT, PER_SM, DF, NW, FULL>;
+    auto *const kern = lean_pass_kernel<R, RB, NT, PER_SM, DF, NW, FULL, SMALL>;
     static int attr_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -160,12 +163,24 @@ int launch_lean_pass(const LaunchCtx &c, const LeanPassArgs &a, const DevPass &h
         return a.nwords <= 480 ? launch_lean_t<float, B64, 256, 2, false, 480, false>(c, a, h, err, errlen)
                                : launch_lean_t<float, B64, 256, 2, false, 2000, false>(c, a, h, err, errlen);
     }
+    // Fewer groups than threads: warps without one stay out of the arithmetic in complex128 (FP64, 10 qubits, 4
+    // layers: 188 -> 125 us, 22 qubits with slabs of 8 bits 33.0 -> 10.4 ms; double-float, the same slabs 9.7 -> 5.8
+    // ms).  complex64 has FP32 issue slots to spare (2.8 -> 1.7 ms there, but 1 % on 10 qubits and 6 % on full slabs
+    // if tested always) and keeps one kernel.
+    const bool narrow = a.stage_bits == B128 - 1;
+    if (h.b - a.stage_bits < (narrow ? 9 : 8)) {
+        if (a.df)
+            return narrow ? launch_lean_t<double, B128 - 1, 512, 1, true, 0, true, true>(c, a, h, err, errlen)
+                          : launch_lean_t<double, B128, 256, 2, true, 0, true, true>(c, a, h, err, errlen);
+        return narrow ? launch_lean_t<double, B128 - 1, 512, 1, false, 0, true, true>(c, a, h, err, errlen)
+                      : launch_lean_t<double, B128, 256, 2, false, 0, true, true>(c, a, h, err, errlen);
+    }
     if (a.df) {
-        if (a.stage_bits == B128 - 1) return launch_lean_t<double, B128 - 1, 512, 1, true, 0, true>(c, a, h, err, errlen);
+        if (narrow) return launch_lean_t<double, B128 - 1, 512, 1, true, 0, true>(c, a, h, err, errlen);
         return a.full ? launch_lean_t<double, B128, 256, 2, true, 0, true>(c, a, h, err, errlen)
                       : launch_lean_t<double, B128, 256, 2, true, 0, false>(c, a, h, err, errlen);
     }
-    if (a.stage_bits == B128 - 1) return launch_lean_t<double, B128 - 1, 512, 1, false, 0, true>(c, a, h, err, errlen);
+    if (narrow) return launch_lean_t<double, B128 - 1, 512, 1, false, 0, true>(c, a, h, err, errlen);
     return launch_lean_t<double, B128, 256, 2, false, 0, true>(c, a, h, err, errlen);
 }
 

@@ -159,9 +159,10 @@ __global__ void __launch_bounds__(NT, 1)
                 if ((base & op.ocmask) == op.ocmask) {
                     if (op.type == OP_STAGE) {
                         const DevStage *st = stages + op.mat;
-                        if (words != nullptr && st->lean_begin >= 0)
-                            run_lean_stage<C, RB>(sm, GlobalWords{words}, uint32_t(st->lean_begin), pool, base, tid);
-                        else run_stage<C, RB>(sm, st, subs, coef, base, tid, NT);
+                        if (words != nullptr && st->lean_begin >= 0) {
+                            if (with_groups(tid, b - RB))
+                                run_lean_stage<C, RB>(sm, GlobalWords{words}, uint32_t(st->lean_begin), pool, base, tid);
+                        } else run_stage<C, RB>(sm, st, subs, coef, base, tid, NT);
                     } else run_smem_op<C>(sm, b, op, coef, base, tid, NT);
                 }
                 __syncthreads();

@@ -656,11 +656,16 @@ __device__ __forceinline__ uint2 condition_index(ulonglong2 cw, uint32_t nl, uin
     return make_uint2(hl, ho);
 }
 
+// Whether some thread of this one's warp has a group of a stage over 2^nrest of them.
+__device__ __forceinline__ bool with_groups(uint32_t tid, int nrest) { return ((tid & ~31u) >> nrest) == 0; }
+
 // Runs the stage whose words start at `at` on the slab in shared memory (addressing: run_stage) and
 // returns the index after its last word.  One group per thread, the caller has at least 2^nrest threads.
 // (With a loop over groups the compiler keeps the 31 address offsets live across it, which costs
 // spills at 128 registers.)  Threads without a group work on a copy of one and store nothing, so that
-// control flow stays the same for the whole warp.
+// control flow stays the same for the whole warp; what they load may be stored by its owner at the same time, and is
+// never used.  In complex128 warps without any group should not come here (with_groups): their copies would
+// take the FP64 pipe as long as real work (10 qubits, 4 layers: 188 us, 125 without; slabs of 8 bits 3.2 times).
 // FULL = false: stages without separable tables, X and half tables, in complex64 without phases too.  The larger set
 // costs the common records registers and moves (layered-28 complex64: 41.2 ms with one set, 37.8 with two).
 template <typename C, int RB, bool FULL = true, typename Words>
