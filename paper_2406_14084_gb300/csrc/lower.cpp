@@ -37,6 +37,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <cstring>
 
 namespace qs {
@@ -153,6 +154,7 @@ struct Builder {
                     }
         t.sep = std::move(groups);
         if (carry_reads() || (!unit && carried())) {
+            t.lift = lift();
             apply_carry_sep(t);
             reset_carry();
         }
@@ -226,6 +228,7 @@ struct Builder {
     {
         // (a carry that is the same for all elements waits for the stage's end)
         if (carry_reads() || (!unit && carried())) {
+            t.lift = lift();
             apply_carry(t);
             reset_carry();
         }
@@ -254,6 +257,8 @@ struct Builder {
         for (uint8_t c : b.dl)
             if (std::find(dl.begin(), dl.end(), c) == dl.end()) dl.push_back(c);
         if (dl.size() > std::max(a.dl.size(), b.dl.size()) && (int)dl.size() > table_bits(plan)) return false;
+        Lift both = a.lift;
+        if (!in_range(both += b.lift)) return false;
         std::vector<int> at(b.dl.size());
         for (size_t j = 0; j < b.dl.size(); ++j) at[j] = int(std::find(dl.begin(), dl.end(), b.dl[j]) - dl.begin());
         grow(a, dl);
@@ -263,6 +268,7 @@ struct Builder {
             for (int e = 0; e < E; ++e) a.tab[(h << RB) | e] = mul(a.tab[(h << RB) | e], b.tab[(hb << RB) | e]);
         }
         a.rd |= b.rd;
+        a.lift = both;
         return true;
     }
     void apply_carry(LeanItem &t) const
@@ -320,7 +326,8 @@ struct Builder {
             return;
         }
         const double det = s00 * s11 - s01 * s10;
-        if (!(std::abs(s11) > 0.0) || !(std::abs(det) > 1e-6 * s11 * s11)) {
+        auto moderate = [](double v) { return std::abs(v) > 0x1p-30 && std::abs(v) < 0x1p30; };
+        if (!moderate(s11) || !moderate(det / s11) || !(std::abs(det) > 1e-6 * s11 * s11)) {
             bad = true;
             return;
         }
@@ -343,7 +350,24 @@ struct Builder {
                 break;
             }
     }
-    // The carried diagonal joins the last table it can be moved back to, or becomes a scaling.
+    Lift lift() const
+    {
+        Lift r;
+        r.e[0] = std::ilogb(carry(0));
+        for (int j = 0; j < RB; ++j)
+            if (d[j][1] != d[j][0]) r.e[1 + j] = std::ilogb(d[j][1] / d[j][0]);
+        return r;
+    }
+    // whether all factors of an item that took these in, and what later records hold instead, stay within FP32 (double-float: also
+    // 2^-48 of them, the last bits of a product)
+    bool in_range(const Lift &t) const
+    {
+        int sum = 0;
+        for (int v : t.e) sum += std::abs(v);
+        return sum < (plan.opt.arith == QS_ARITH_DF ? 40 : 90);
+    }
+    // The carried diagonal joins the last table it can be moved back to, or becomes a scaling: also where a table
+    // that many of them have joined would leave the range of FP32.
     void flush_carry()
     {
         if (!carried()) return;
@@ -357,7 +381,8 @@ struct Builder {
             }
             if (it.op == L_CX && d[it.j][0] != d[it.j][1]) break;
         }
-        if (!found) {
+        Lift after = lift();
+        if (!found || !in_range(after += items[t].lift)) {
             LeanItem sc;
             sc.op = L_SCALE;
             sc.scale.resize(E);
@@ -375,6 +400,7 @@ struct Builder {
                         items[i].y[j] /= r;  // D L = (D L D^-1) D
                         items[i].x[j] *= r;
                     }
+        items[t].lift = after;
         if (items[t].op == L_SEP) apply_carry_sep(items[t]);
         else apply_carry(items[t]);
         reset_carry();
@@ -449,6 +475,11 @@ struct Builder {
         case SB_PHASE: {
             const cd p = M[0];
             if (!ctl && p.imag() == 0.0) {
+                // (rotations alone stay just beyond 2^-64; matrices scaled further keep their order of factors)
+                if (!(std::abs(p.real()) > 0x1p-68 && std::abs(p.real()) < 0x1p68)) {
+                    bad = true;
+                    break;
+                }
                 d[0][0] *= p.real();
                 d[0][1] *= p.real();
                 break;

@@ -15,6 +15,16 @@ struct SepGroup {
     std::vector<cd> tab;
 };
 
+// Exponents of carried factors: that of slot 0, then of each register bit's ratio.
+struct Lift {
+    int e[7] = {};
+    Lift &operator+=(const Lift &o)
+    {
+        for (int j = 0; j < 7; ++j) e[j] += o.e[j];
+        return *this;
+    }
+};
+
 // One record of a lowered stage, in FP64; lower_stages() writes it in the state precision.
 struct LeanItem {
     LeanOp op = L_ROTA;
@@ -28,6 +38,7 @@ struct LeanItem {
     std::vector<uint8_t> dl;        // L_TABLE: condition bits (DevSub::dl codes)
     std::vector<SepGroup> sep;      // L_SEP
     std::vector<double> scale;      // L_SCALE: 2^RB real factors
+    Lift lift;                      // L_TABLE, L_SEP: the carried factors that they took in
     uint32_t rd = 0;                // diagonals: register bits the factors may depend on
     uint32_t m32 = 0;               // L_PHASE: register elements the phase p acts on
     cd p = 1.0;

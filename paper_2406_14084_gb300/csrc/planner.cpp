@@ -653,6 +653,9 @@ bool controlled_phase(const CGate &g, cd &phase)
 // the larger tables).
 int default_merge_bits(const Plan &plan) { return plan.dt == QS_C128 && plan.opt.arith == QS_ARITH_FP64 ? 10 : 6; }
 
+// A stage scalar that has to stay where it is (factor_stage_rotations).
+bool far_scalar(double v) { return !(std::abs(v) > 0x1p-64 && std::abs(v) < 0x1p64); }
+
 void merge_stage_diagonals(Plan &plan, int s0, int RB, Coefs &cf)
 {
     const int kMergeCondBits = plan.opt.merge_bits > 0 ? std::min(plan.opt.merge_bits, 10) : default_merge_bits(plan);
@@ -668,7 +671,8 @@ void merge_stage_diagonals(Plan &plan, int s0, int RB, Coefs &cf)
         }
     };
     auto is_diag = [](const DevSub &s) { return s.type == SB_PHASE || s.type == SB_DIAG; };
-    auto eligible = [kMergeCondBits](const DevSub &s) {
+    auto eligible = [kMergeCondBits, &plan](const DevSub &s) {
+        if (s.type == SB_PHASE && !(s.scm | s.lcm | s.ocm) && far_scalar(std::abs(plan.coef[s.mat]))) return false;
         return (s.type == SB_PHASE && __builtin_popcount(s.lcm) + __builtin_popcountll(s.ocm) <= kMergeCondBits) ||
                (s.type == SB_DIAG && s.ndl == 0);
     };
@@ -799,7 +803,9 @@ void merge_stage_diagonals(Plan &plan, int s0, int RB, Coefs &cf)
 //   otherwise:       M = m01 [[m00/m01, 1], [m10/m01, m11/m01]],  m10/m01 = +1 or -1  (A, AM)
 // so every ratio is at most 1 in magnitude.  The scalars of all factored subs are collected into
 // one scalar sub of the stage (a diagonal that reads no bit), which the diagonal merge that
-// follows folds into a table where one exists.  The matrices are FP64 ratios of the gate's own
+// follows folds into a table where one exists.  Where their product leaves 2^-64 .. 2^64 it becomes a scalar of
+// its own at that place, which no merge moves (far_scalar): the amplitudes grow by its inverse meanwhile, and
+// FP32 holds neither beyond 2^126 (5 qubits, 200 layers in one stage read 0 or NaN).  The matrices are FP64 ratios of the gate's own
 // entries (Eq. 2-3 reassociated), so results change only by rounding.
 void factor_stage_rotations(Plan &plan, int s0, Coefs &cf)
 {
@@ -817,6 +823,13 @@ void factor_stage_rotations(Plan &plan, int s0, Coefs &cf)
     double sigma = 1.0;
     std::vector<DevSub> out;
     out.reserve(in.size() + cand + 1);
+    auto scalar_sub = [&](double v) {
+        DevSub sc;
+        std::memset(&sc, 0, sizeof sc);
+        sc.type = SB_PHASE;
+        sc.mat = cf.push(std::vector<cd>{cd(v)});
+        return sc;
+    };
     for (const DevSub &sb : in) {
         if (sb.type != SB_G1R || (sb.scm | sb.lcm | sb.ocm)) {
             out.push_back(sb);
@@ -849,12 +862,12 @@ void factor_stage_rotations(Plan &plan, int s0, Coefs &cf)
         f.mat = cf.push(std::vector<cd>{cd(x), cd(y)});
         out.push_back(f);
         sigma *= d;
+        if (far_scalar(sigma)) {
+            out.push_back(scalar_sub(sigma));
+            sigma = 1.0;
+        }
     }
-    DevSub sc;
-    std::memset(&sc, 0, sizeof sc);
-    sc.type = SB_PHASE;
-    sc.mat = cf.push(std::vector<cd>{cd(sigma)});
-    out.push_back(sc);
+    out.push_back(scalar_sub(sigma));
     plan.subs.resize(s0);
     plan.subs.insert(plan.subs.end(), out.begin(), out.end());
 }

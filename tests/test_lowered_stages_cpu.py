@@ -88,3 +88,16 @@ def test_separable_records_from_fused_tables(compare, n, form):
         worst, count = compare(W.qaoa_complete(n, 2, seed), n, **FORMS[form][0])
         assert count[2] > 0
         assert worst <= tol, (seed, worst)
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("n", [4, 5, 6])
+@pytest.mark.parametrize("real", [False, True])
+def test_long_stages(compare, real, n, form):
+    """Thousands of rotations in one stage: their common factor, below 2^-126, has to stay within FP32."""
+    opts, tol = FORMS[form]
+    rng = W.SplitMix64(n)
+    gates = [Gate("T", (0,))] + [Gate("RY", (rng.below(n),), (), (rng.angle(),)) for _ in range(3000)] if real \
+        else W.layered(n, 500, n)
+    worst, _ = compare(gates, n, fuse_width=0 if real else 2, **opts)
+    assert worst <= tol * 10  # ten times the records of the other tests
