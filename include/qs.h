@@ -291,11 +291,12 @@ qs_status qs_probs_noalloc(const void *dev_amp, int n, qs_dtype dt, const int *q
 qs_status qs_sample(qs_state *s, const double *u, size_t shots, uint64_t *host_out);
 
 /* host_out[0] = Re sum_t coeff_t <psi|P_t|psi>, host_out[1] = its imaginary part (zero up to
- * rounding for Hermitian sums).  Terms are grouped by X mask (at most 256 per group).  Groups of four
- * or more terms on 16 or more qubits cost one read of the state each, through Walsh-Hadamard
- * tiles, whatever the group's size; smaller groups share reads where their X masks fit the bits of
- * one shared-memory tile (13 qubits, complex128 12), and take one read each otherwise.  FP64
- * accumulation across tiles (complex64 states: FP32 within a tile).  Synchronises. */
+ * rounding for Hermitian sums).  Terms are grouped by X mask (at most 256 per group).  Groups with a
+ * nonzero X mask and at most 8 terms share reads of the state where their X masks fit the bits of one
+ * shared-memory tile (13 qubits, complex128 12) and that costs less than a pass each.  Of the others,
+ * groups of four or more terms on 16 or more qubits cost one read each, through Walsh-Hadamard tiles,
+ * whatever the group's size, and smaller ones one pass each.  FP64 accumulation across tiles
+ * (complex64 states: FP32 within a tile, over at most four X masks or eight terms).  Synchronises. */
 qs_status qs_expect_pauli_sum(qs_state *s, const qs_pauli_term *terms, size_t nterms,
                               double *host_out);
 

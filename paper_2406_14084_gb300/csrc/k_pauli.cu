@@ -37,7 +37,9 @@ struct PauliTerm {
 };
 struct PauliGroup {
     uint32_t xm;     // tile-local
-    uint16_t piv, t0, tmid, t1;  // terms [t0, tmid) use Re v, [tmid, t1) Im v
+    uint8_t piv;     // its highest bit
+    uint8_t flush;   // the FP32 sums go to FP64 after this mask
+    uint16_t t0, tmid, t1;  // terms [t0, tmid) use Re v, [tmid, t1) Im v
 };
 struct PauliTile {
     int lo, nhi, ngroups, nterms;
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 3) pauli_tile_kernel(const typename 
                 values(true);
                 terms(q.tmid, q.t1);
             }
-            if (sizeof(R) == 4 && (g & 3) == 3) {  // FP32 sums stay as short as with one pass per mask (1.27 -> 1.33 ms)
+            if (sizeof(R) == 4 && q.flush) {
                 acc += (double)facc;
                 facc = 0;
             }
@@ -193,9 +195,10 @@ int launch_t(const LaunchCtx &c, const PauliTile *d, const PauliTile &h, int b, 
 
 size_t pauli_tile_bytes() { return sizeof(PauliTile); }
 
-// Takes the groups listed in `todo` (indices into groups; each has an X mask) that fit the next tile and
-// removes them from it; fills h and returns the tile's bits, or 0 if the first one fits no tile.
-int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, std::vector<int> &todo, void *h)
+// Moves the groups listed in `todo` (indices into groups; each has an X mask) that fit the next tile to `take`,
+// fills h and returns the tile's bits; 0 if none of them fits a tile.
+int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, std::vector<int> &todo,
+                    std::vector<int> &take, void *h)
 {
     PauliTile &p = *static_cast<PauliTile *>(h);
     std::memset(&p, 0, sizeof p);
@@ -203,7 +206,7 @@ int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, 
     const int lo = std::min(c.dt == QS_C64 ? 4 : 3, bmax);
     uint64_t bits = (1ull << lo) - 1;
     std::vector<int> left;
-    std::vector<int> take;
+    take.clear();
     size_t nterms = 0;
     for (int gi : todo) {
         const PauliXGroup &g = groups[gi];
@@ -234,11 +237,12 @@ int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, 
             if ((m >> q & 1) && local_of[q] >= 0) r |= 1u << local_of[q];
         return r;
     };
+    int since = 0;
     for (int gi : take) {
         const PauliXGroup &g = groups[gi];
         PauliGroup &G = p.g[p.ngroups++];
         G.xm = local(g.xm);
-        G.piv = uint16_t(31 - __builtin_clz(G.xm));
+        G.piv = uint8_t(31 - __builtin_clz(G.xm));
         G.t0 = uint16_t(p.nterms);
         for (int odd = 0; odd < 2; ++odd) {
             for (size_t t = 0; t < g.zm.size(); ++t) {
@@ -258,6 +262,13 @@ int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, 
             if (!odd) G.tmid = uint16_t(p.nterms);
         }
         G.t1 = uint16_t(p.nterms);
+        // FP32 sums of at most 8 terms or 4 masks, each of 16 pairs (a pass per mask adds 32 pairs in FP32; the chain
+        // takes 1.27 ms without, 1.33 so)
+        since += std::max(2, G.t1 - G.t0);
+        if (since >= 8) {
+            G.flush = 1;
+            since = 0;
+        }
     }
     todo = std::move(left);
     return b;

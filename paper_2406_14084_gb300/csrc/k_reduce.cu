@@ -833,27 +833,47 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
     // One host image per launch, 32 launches between waits (at most 360 KiB).
     auto wait = [st] { cudaStreamSynchronize(st); };
     StagingRing<decltype(wait)> staging(std::max({pauli_tile_bytes(), sizeof(TermGroup), sizeof(WhtTerms)}), 32, wait);
-    if (cudaMemsetAsync(res, 0, 2 * sizeof(double), st) != cudaSuccess) return cuda_fail("expect memset", err, errlen);
+    if (groups.empty()) {
+        h_out[0] = h_out[1] = 0.0;
+        return QS_OK;
+    }
+    bool first = true;  // the first launch's sums are stored, the others' added
     // X masks with few terms share reads of the state (k_pauli.cu).  A term costs a tile pass about 2
     // operations per pair of amplitudes, so up to 8 terms per mask are well below a pass of their own.
+    // Whether a tile pass is taken depends on what it replaces.  One mask alone: from 18 qubits on it is read
+    // once and not twice (complex64, 27 qubits, 1 term: 1054 -> 403 us; below, 40 us either way).  Masks that
+    // all have Walsh-Hadamard tiles of their own (4 terms, 16 qubits): in complex64 those run at HBM rate (27
+    // qubits 227 us, against 451 for a tile pass and about 130 for each further mask), so from four masks on;
+    // in complex128 the transform is FP64 work and the tile pass is ahead (26 qubits, 8 terms: 1488 -> 1230
+    // us).  Small complex128 states: up to 16 CTAs, each bound by FP64 issue, 2.5 us a term against 6 us for
+    // a launch (14 qubits, 8 terms: 57 us, 41 on its own).
+    auto worthwhile = [&](const std::vector<int> &take) {
+        size_t nt = 0, light = 0;
+        for (int g : take) {
+            nt += groups[g].zm.size();
+            light += groups[g].zm.size() < 4 || c.n < 16;
+        }
+        const bool c64 = c.dt == QS_C64;
+        if (take.size() == 1 && light) return c.n >= 18;
+        if (!c64) return c.n >= 17 || 2 * nt <= 5 * take.size();
+        return light > 0 || take.size() >= 4;
+    };
     std::vector<int> tiles;
     std::vector<char> done(groups.size(), 0);
     for (size_t g = 0; g < groups.size(); ++g)
         if (groups[g].xm != 0 && groups[g].zm.size() <= 8) tiles.push_back(int(g));
     while (!tiles.empty()) {
-        const std::vector<int> before = tiles;
+        std::vector<int> take;
         void *const htile = staging.next();
-        const int b = pauli_tile_plan(c, groups, tiles, htile);
-        if (b == 0) {
-            tiles.erase(tiles.begin());  // more X bits than a tile holds: a pass of its own below
-            continue;
-        }
-        for (int g : before) done[g] = 1;
-        for (int g : tiles) done[g] = 0;
+        const int b = pauli_tile_plan(c, groups, tiles, take, htile);
+        if (b == 0) break;  // more X bits than a tile holds, all of them: passes of their own below
+        if (!worthwhile(take)) continue;
+        for (int g : take) done[g] = 1;
         if (cudaMemcpyAsync(dtile, htile, pauli_tile_bytes(), cudaMemcpyHostToDevice, st) != cudaSuccess)
             return cuda_fail("expect upload", err, errlen);
         const int nblk = launch_pauli_tile(c, dtile, htile, b, part, kRedBlocksMax);
-        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
+        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, !first);
+        first = false;
         int rc = cuda_fail("expect launch", err, errlen);
         if (rc) return rc;
     }
@@ -907,7 +927,8 @@ int launch_expect(const LaunchCtx &c, const uint64_t *xm, const uint64_t *zm, co
                 expect_kernel<double><<<blocks, kRedThreads, 0, st>>>((const double2 *)c.amp, N, dgrp,
                                                                       part);
         }
-        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, true);
+        finish_kernel<<<1, kRedThreads, 0, st>>>(part, nblk, nblk, res, !first);
+        first = false;
         int rc = cuda_fail("expect launch", err, errlen);
         if (rc) return rc;
     }

@@ -276,7 +276,8 @@ struct PauliXGroup {
     std::vector<double> c;
 };
 size_t pauli_tile_bytes();
-int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, std::vector<int> &todo, void *h_tile);
+int pauli_tile_plan(const LaunchCtx &c, const std::vector<PauliXGroup> &groups, std::vector<int> &todo,
+                    std::vector<int> &take, void *h_tile);
 // returns the number of blocks, each of which leaves one partial sum
 int launch_pauli_tile(const LaunchCtx &c, const void *d_tile, const void *h_tile, int b, double *part, int max_blocks);
 int launch_set_basis(const LaunchCtx &c, uint64_t x, char *err, size_t errlen);
