@@ -46,7 +46,9 @@ namespace {
 
 // Condition bits up to which a table grows to take in a conditional phase.  A sign costs three
 // integer instructions per element as a record of its own; FP32 tables double in size per bit.
-int table_bits(const Plan &plan) { return plan.dt == QS_C128 && plan.opt.arith == QS_ARITH_FP64 ? 10 : 5; }
+// (qs_options.merge_bits limits what is put together here as it does the planner's own tables.)
+int limited(const Plan &plan, int bits) { return plan.opt.merge_bits > 0 ? std::min(bits, plan.opt.merge_bits) : bits; }
+int table_bits(const Plan &plan) { return limited(plan, plan.dt == QS_C128 && plan.opt.arith == QS_ARITH_FP64 ? 10 : 5); }
 
 // Product of finite numbers (operator* of std::complex also checks for NaN, several times slower).
 inline cd mul(const cd &a, const cd &b)
@@ -426,14 +428,14 @@ struct Builder {
         case SB_G1NM: add_real(sb.j0, 1.0, M[0].real(), M[1].real(), -1.0); break;
         case SB_G1A: add_real(sb.j0, M[0].real(), 1.0, 1.0, M[1].real()); break;
         case SB_G1AM: add_real(sb.j0, M[0].real(), 1.0, -1.0, M[1].real()); break;
-        case SB_G1R:
-            if (ctl) bad = true;
+        case SB_G1R:  // (factor = 1 keeps full matrices, euler = 1 complex ones: the general engine's)
+            if (ctl || plan.opt.factor == 1) bad = true;
             else add_real(sb.j0, M[0].real(), M[1].real(), M[2].real(), M[3].real());
             break;
         case SB_G1: {
             // complex 2x2: phase, real rotation, phase (the planner's Z-Y-Z form)
             const double c = std::abs(M[0]), s = std::abs(M[2]);
-            if (ctl || c < 1e-6 || s < 1e-6) {
+            if (ctl || plan.opt.factor == 1 || plan.opt.euler == 1 || c < 1e-6 || s < 1e-6) {
                 bad = true;
                 break;
             }
@@ -733,7 +735,7 @@ uint32_t sub_targets(const DevSub &s)
     }
 }
 
-constexpr int kSepBits = 8;      // condition bits per group
+constexpr int kSepBits = 8;      // condition bits per group, at most merge_bits
 constexpr size_t kSepGroups = 24;
 
 // The stage with its separable conditional diagonals collected at as few places as possible; each place
@@ -780,6 +782,7 @@ bool lower_regrouped(const Plan &plan, const DevSub *sub, int ns, int RB, Builde
         }
     }
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return conds[x].hi < conds[y].hi; });
+    const int most = limited(plan, kSepBits);
     std::vector<std::vector<SepGroup>> at(m + 1);
     std::vector<uint32_t> at_rd(m + 1, 0);
     for (int i : order) {
@@ -791,7 +794,7 @@ bool lower_regrouped(const Plan &plan, const DevSub *sub, int ns, int RB, Builde
                 conds[k].point = p;
                 in.push_back(k);
             }
-        // groups of at most kSepBits conditions: the most widely used orders first, by condition code
+        // groups of at most `most` conditions: the most widely used orders first, by condition code
         std::stable_sort(in.begin(), in.end(), [&](int x, int y) {
             const auto &a = conds[x].f.dl, &c = conds[y].f.dl;
             return std::lexicographical_compare(a.begin(), a.end(), c.begin(), c.end());
@@ -801,11 +804,11 @@ bool lower_regrouped(const Plan &plan, const DevSub *sub, int ns, int RB, Builde
         for (int k : in) {
             const std::vector<uint8_t> &dl = conds[k].f.dl;
             size_t best = groups.size();
-            int fewest = kSepBits + 1;
+            int fewest = most + 1;
             for (size_t g = 0; g < groups.size(); ++g) {
                 int extra = 0;
                 for (uint8_t c : dl) extra += std::find(groups[g].dl.begin(), groups[g].dl.end(), c) == groups[g].dl.end();
-                if (extra < fewest && (int)groups[g].dl.size() + extra <= std::max<int>(kSepBits, (int)dl.size())) {
+                if (extra < fewest && (int)groups[g].dl.size() + extra <= std::max<int>(most, (int)dl.size())) {
                     fewest = extra;
                     best = g;
                 }

@@ -70,19 +70,55 @@ double held(double x, qs_dtype dt, bool df)
     return (double)h + (double)(float)(x - (double)h);
 }
 
+// The plan of a circuit, or false.
+bool plan_of(const qs_gate *g, size_t ng, int n, const qs_options *opt, Plan &p)
+{
+    std::vector<CGate> cg;
+    std::string err;
+    return !canonicalize(g, ng, n, cg, err) && !build_plan(cg, n, (qs_dtype)opt->dtype, *opt, p, err);
+}
+
 }  // namespace
+
+// most: condition bits of a lowered table, of a separable group, of a sub-op of the plan (before and after the
+// planner's merges); lowered stages with a 2x2 matrix; stages with one.
+extern "C" int lowered_widths(const qs_gate *g, size_t ng, int n, const qs_options *opt, int64_t *most)
+{
+    Plan p;
+    if (!plan_of(g, ng, n, opt, p)) return -1;
+    auto conditions = [](const DevSub &s) -> int64_t {
+        if (s.type == SB_DIAG) return s.ndl;
+        return s.type == SB_PHASE ? __builtin_popcount(s.lcm) + __builtin_popcountll(s.ocm) : 0;
+    };
+    for (const DevSub &s : p.raw_subs) most[2] = std::max(most[2], conditions(s));
+    for (const DevSub &s : p.subs) most[2] = std::max(most[2], conditions(s));
+    for (const DevStage &st : p.stages) {
+        LeanStage ls;
+        lower_stage(p, st, p.stage_bits, ls);
+        bool matrix = false;
+        for (int i = st.sub_begin; i < st.sub_end; ++i) {
+            const int t = p.subs[i].type;
+            matrix |= t != SB_PHASE && t != SB_DIAG && t != SB_X && t != SB_SWAP;
+        }
+        most[4] += matrix;
+        if (!ls.ok) continue;
+        most[3] += matrix;
+        for (const LeanItem &it : ls.items) {
+            if (it.op == L_TABLE) most[0] = std::max<int64_t>(most[0], it.dl.size());
+            for (const SepGroup &q : it.sep) most[1] = std::max<int64_t>(most[1], q.dl.size());
+        }
+    }
+    return 0;
+}
 
 // count: stages, lowered stages, separable records, records in all.  Returns the largest difference of an
 // amplitude relative to the largest amplitude of its group (inf for a NaN), or -1 on a bad circuit.
 extern "C" double lowered_difference(const qs_gate *g, size_t ng, int n, const qs_options *opt, int64_t *count)
 {
-    std::vector<CGate> cg;
-    std::string err;
-    if (canonicalize(g, ng, n, cg, err)) return -1.0;
     const qs_dtype dt = (qs_dtype)opt->dtype;
     const bool df = dt == QS_C128 && opt->arith == QS_ARITH_DF;
     Plan p;
-    if (build_plan(cg, n, dt, *opt, p, err)) return -1.0;
+    if (!plan_of(g, ng, n, opt, p)) return -1.0;
     const int RB = p.stage_bits;
     const uint32_t E = 1u << RB;
     std::mt19937_64 rng(1);

@@ -24,24 +24,32 @@ FORMS = {"c64": (dict(dtype=qs.QS_C64), 1e-5), "c128": (dict(dtype=qs.QS_C128), 
 
 
 @pytest.fixture(scope="module")
-def compare(tmp_path_factory):
+def host(tmp_path_factory):
     qs.lib()
     so, lib = qs.library_path(), str(tmp_path_factory.mktemp("lowered") / "lowered_stages.so")
     pkg = os.path.dirname(os.path.abspath(qs.__file__))
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(pkg, "..", "include"), "-I",
                     os.path.join(pkg, "csrc"), os.path.join(HERE, "lowered_stages.cpp"), so, "-o", lib,
                     "-Wl,-rpath," + os.path.dirname(so)], check=True)
-    fn = ctypes.CDLL(lib).lowered_difference
-    fn.restype = ctypes.c_double
+    dll = ctypes.CDLL(lib)
+    dll.lowered_difference.restype = ctypes.c_double
+    return dll
 
+
+def call(fn, numbers, gates, n, **kw):
+    arr, keep = qs.marshal_gates(gates)
+    opts, out = qs.options(**kw), (ctypes.c_int64 * numbers)()
+    rc = fn(arr, ctypes.c_size_t(len(gates)), n, ctypes.byref(opts), out)
+    del keep
+    assert rc >= 0
+    return rc, tuple(out)
+
+
+@pytest.fixture(scope="module")
+def compare(host):
     def run(gates, n, **kw):
         """Largest difference and (stages, lowered stages, separable records, records)."""
-        arr, keep = qs.marshal_gates(gates)
-        opts, count = qs.options(**kw), (ctypes.c_int64 * 4)()
-        worst = fn(arr, ctypes.c_size_t(len(gates)), n, ctypes.byref(opts), count)
-        del keep
-        assert worst >= 0.0
-        return worst, tuple(count)
+        return call(host.lowered_difference, 4, gates, n, **kw)
 
     return run
 
@@ -101,3 +109,25 @@ def test_long_stages(compare, real, n, form):
         else W.layered(n, 500, n)
     worst, _ = compare(gates, n, fuse_width=0 if real else 2, **opts)
     assert worst <= tol * 10  # ten times the records of the other tests
+
+
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("merge", [1, 2, 4, 6, 8])
+def test_merge_bits_limits_what_is_put_together(host, merge, form):
+    """Tables and separable groups read at most merge_bits conditions, unless one diagonal alone reads more."""
+    for gates, n in ((W.qft(16), 16), (pairs(13, 3, None), 13), (W.qaoa_complete(14, 2, 1), 14)):
+        for fuse in (0, 2):
+            _, most = call(host.lowered_widths, 5, gates, n, merge_bits=merge, fuse_width=fuse, slab_bits=9, **FORMS[form][0])
+            assert max(most[0], most[1]) <= max(merge, most[2])
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_kept_matrices_stay_on_the_general_engine(host, form):
+    """factor = 1 keeps full 2x2 matrices and euler = 1 complex ones: no stage with one is lowered."""
+    opts = FORMS[form][0]
+    _, on = call(host.lowered_widths, 5, W.layered(12, 4, 3), 12, fuse_width=1, **opts)
+    assert on[3] == on[4] > 0
+    _, off = call(host.lowered_widths, 5, W.layered(12, 4, 3), 12, fuse_width=1, factor=1, **opts)
+    assert off[3] == 0 < off[4]
+    _, off = call(host.lowered_widths, 5, W.layered(12, 4, 3), 12, fuse_width=1, euler=1, **opts)
+    assert off[3] < off[4]
