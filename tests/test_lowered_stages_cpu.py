@@ -131,3 +131,18 @@ def test_kept_matrices_stay_on_the_general_engine(host, form):
     assert off[3] == 0 < off[4]
     _, off = call(host.lowered_widths, 5, W.layered(12, 4, 3), 12, fuse_width=1, euler=1, **opts)
     assert off[3] < off[4]
+
+
+def test_batch_circuits_lower_throughout(compare):
+    """The circuits of test_gpu_batch_lean_sizes.py have register stages only, and all of them are lowered."""
+    import test_gpu_batch_lean_sizes as B
+
+    for slab, width in B.CASES:
+        for n, gates in B.circuits_of(width):
+            opts = dict(dtype=qs.QS_C64, slab_bits=slab, stage_bits=width)
+            _, count = compare(gates, n, **opts)
+            assert 0 < count[0] == count[1], (n, slab, width)
+            plan = qs.qs_fuse(gates, n, qs.options(**opts))
+            info = qs.qs_plan_info_get(plan)
+            qs.qs_plan_destroy(plan)
+            assert info["smem_ops"] == 0, (n, slab, width)
