@@ -88,7 +88,7 @@ PAPER_GATES_PER_S = {"qaoa31_c128": 2511 / 17.5, "qft31_c128": 496 / 3.6}
 # per SM per clock (128 FP32, 2 FP64) x 2 flops per FMA.
 ALU_PEAK_TFLOPS = {"c64": 152 * 2.07e9 * 128 * 2 / 1e12, "c128": 152 * 2.07e9 * 2 * 2 / 1e12}
 
-TRAFFIC_SOURCES = ("k_lean.cu", "lean_stage.cuh", "slab_common.cuh", "dev_common.cuh", "df_arith.cuh")
+TRAFFIC_SOURCES = ("k_lean.cu", "lean_stage.cuh", "slab_common.cuh", "dev_common.cuh", "df_arith.cuh", "qs_internal.h")
 
 
 def slab_kernel_hash() -> str:
@@ -120,6 +120,15 @@ def circuit_flops_per_amp(gates) -> float:
         else:
             f += 8.0 * 2 ** k * sel
     return f
+
+
+def pass_kernels(info: dict) -> str:
+    """The kernels that run a plan's passes: in place, general, or both."""
+    lean, general = info["lean_passes"], info["passes"] + info["remaps"] - info["lean_passes"]
+    names = [k for k, passes in (("lean_pass_kernel", lean), ("slab_pass_kernel", general)) if passes]
+    if info["unblocked"]:
+        names.append("unblocked_kernel")
+    return " + ".join(names) or "none"
 
 
 def measured_traffic(n: int, dtype: str):
@@ -1054,10 +1063,11 @@ def run_gpu(args, w, ws, rank, local):
     exec_flops_amp = 2.0 * float(plan_fma_per_amp)
     alu_tflops = exec_flops_amp * (1 << n) * args.steps / (pass_ms_total / 1e3) / 1e12
     algo_flops_amp = circuit_flops_per_amp(gates)
-    traffic = measured_traffic(n, w["dtype"])
+    kernels = pass_kernels(info)
+    traffic = measured_traffic(n, w["dtype"]) if kernels == "lean_pass_kernel" else None  # captured on it
     roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
-            "kernel": "lean_pass_kernel", "peak_source": peaks["source"],
+            "kernel": kernels, "peak_source": peaks["source"],
             "avg_launch_ms": dom_ms, "bytes_per_launch": pass_bytes}
     tc_roof = None
     if st["tc_gates"] and st["tc_ms"] > pass_ms_total:
@@ -1074,7 +1084,7 @@ def run_gpu(args, w, ws, rank, local):
                    "peak_source": "BF16 dense, " + peaks["source"]}
     alu_peak = ALU_PEAK_TFLOPS["c64" if dtype == qs.QS_C64 else "c128"]
     roof_alu = {"bound": "alu", "achieved": alu_tflops, "peak": alu_peak, "unit": "TFLOP/s",
-                "frac": alu_tflops / alu_peak, "traffic": traffic, "kernel": "lean_pass_kernel",
+                "frac": alu_tflops / alu_peak, "traffic": traffic, "kernel": kernels,
                 "avg_launch_ms": dom_ms,
                 "flops_per_launch": exec_flops_amp * (1 << n) / max(1, passes_per_step),
                 "algorithmic_flops_per_amp": exec_flops_amp,

@@ -158,7 +158,8 @@ typedef struct {
     double judge_ms_learned;     /* measured device time of the first learned apply (0 = none) */
     double judge_ms_greedy;      /* measured device time of the first greedy apply (0 = none) */
     int32_t using_greedy;  /* 1 once the judge found the greedy plan faster */
-    int32_t pad_;
+    int32_t lean_passes;   /* passes whose stages all run on the in-place engine; the others take the
+                              general one */
 } qs_plan_info;
 
 /* Per-state counters, accumulated since creation or the last qs_stats_reset.  The *_ms fields

@@ -164,6 +164,15 @@ struct qs_plan {
     std::vector<DevStage> stages;
     LeanImage image;
     bool lowered = false;
+    int lean_passes = 0;  // passes that the in-place kernel runs
+    // All of the pass's ops are lowered stages.
+    bool lean(const DevPass &P) const
+    {
+        if (P.has_perm || P.op_begin == P.op_end) return false;
+        for (int o = P.op_begin; o < P.op_end; ++o)
+            if (p.ops[o].type != OP_STAGE || stages[p.ops[o].mat].lean_begin < 0) return false;
+        return true;
+    }
     void lower()
     {
         if (lowered) return;
@@ -171,6 +180,8 @@ struct qs_plan {
         image = LeanImage{};
         lower_stages(p, p.dt, p.dt == QS_C128 && p.opt.arith == QS_ARITH_DF, stages, image);
         lowered = true;
+        lean_passes = 0;
+        for (const DevPass &P : p.passes) lean_passes += lean(P);
     }
     ~qs_plan()
     {
@@ -228,9 +239,7 @@ qs_status upload(qs_plan *pl, qs_dtype dt, qs_state *borrow)
     bool general = false;
     for (size_t i = 0; i < p.passes.size(); ++i) {
         const DevPass &P = p.passes[i];
-        bool lean = !P.has_perm && P.op_begin < P.op_end;
-        for (int o = P.op_begin; lean && o < P.op_end; ++o)
-            lean = p.ops[o].type == OP_STAGE && stages[p.ops[o].mat].lean_begin >= 0;
+        const bool lean = pl->lean(P);
         if (lean) {  // the stages of a pass, and so their words, are consecutive
             const DevStage &s0 = stages[p.ops[P.op_begin].mat], &s1 = stages[p.ops[P.op_end - 1].mat];
             d.lean[i].begin = s0.lean_begin;
@@ -792,6 +801,7 @@ qs_status qs_plan_info_get(const qs_plan *p, qs_plan_info *out)
     out->greedy_predicted_ms = p->greedy_pred_ms;
     out->judge_ms_learned = p->judge_ms[0];
     out->judge_ms_greedy = p->judge_ms[1];
+    out->lean_passes = p->lean_passes;
     out->using_greedy = (p->alt && p->use_alt) ? 1 : 0;
     return QS_OK;
 }

@@ -72,7 +72,7 @@ class QsPlanInfo(ctypes.Structure):
                 ("judge_state", ctypes.c_int32), ("predicted_ms", ctypes.c_double),
                 ("greedy_predicted_ms", ctypes.c_double), ("judge_ms_learned", ctypes.c_double),
                 ("judge_ms_greedy", ctypes.c_double), ("using_greedy", ctypes.c_int32),
-                ("pad_", ctypes.c_int32)]
+                ("lean_passes", ctypes.c_int32)]
 
 
 QS_PLAN_FEATURES = 28
