@@ -8,8 +8,8 @@
 // pass program into the second slot while the slab of this one is under way, so the queue's latency
 // (an atomic and three dependent reads) is off the path.  64 circuits of 10-20 qubits: 1.32 ms (one CTA
 // with two slabs and a producer warp: 1.99); 300 of 10-15: 750 -> 377 us; 8 of 14-20: 1160 -> 558 us.
-// complex128 stays on the general engine: FP64 work gains nothing from a second CTA on the SM
-// (59 circuits of 10-15 qubits: 988 us there, 1328 us here).
+// complex64 only: FP64 work gains nothing from a second CTA on the SM, so complex128 stays on the general
+// engine (59 circuits of 10-15 qubits: 991 us there, in place 1063 us with one CTA per SM and 1328 with two).
 //
 // A CTA looks at the next item only after this one is stored, and an item waits only for items before
 // it in the queue: the earliest unfinished item can always run.  The wait is bounded.
@@ -24,6 +24,7 @@ namespace qs {
 namespace {
 
 constexpr uint32_t kSpinLimit = 1u << 23;
+constexpr int kMaxBits = 13;  // 64 KiB of slab
 
 struct __align__(16) LeanSlot {
     uint64_t seg_lo[64], seg_hi[64];  // gather tables of the item's pass, in 16-byte vectors
@@ -55,14 +56,10 @@ struct NearWords {
     __device__ __forceinline__ ulonglong2 bulk(uint32_t i) const { return p[i]; }
 };
 
-template <typename C>
-__device__ __forceinline__ uint32_t chunk_of(uint32_t v)
-{
-    return sizeof(C) == 8 ? (swz<1>(v << 1) >> 1) : swz<2>(v);
-}
+// 16-byte chunk of shared memory that holds amplitudes 2 v and 2 v + 1 of the slab
+__device__ __forceinline__ uint32_t chunk_of(uint32_t v) { return swz<1>(v << 1) >> 1; }
 
 // One warp: the next slab (of the same run, or the first of the next queue item) into slot Z.
-template <typename C>
 __device__ __forceinline__ void fetch(LeanSlot &Z, const LeanSlot *prev, const BatchArgs &a, ulonglong2 *wbuf, uint32_t wcap, uint32_t lane)
 {
     if (lane == 0) {
@@ -90,14 +87,13 @@ __device__ __forceinline__ void fetch(LeanSlot &Z, const LeanSlot *prev, const B
         const ulonglong2 *w = static_cast<const ulonglong2 *>(a.words) + Z.prog.begin;
         for (uint32_t i = lane; i < Z.prog.nwords; i += 32) cp_async16(smem_addr(wbuf + i), w + i);
     }
-    constexpr int kLog16 = (sizeof(C) == 8) ? 1 : 0;
     const int lo = Z.pass.lo, nhi = Z.pass.nhi;
     for (uint32_t j = lane; j < 128; j += 32) {
         const uint32_t x = j & 63, sh = (j < 64) ? 0 : 6;
         uint64_t o = 0;
         for (int m = 0; m < 6; ++m)
             if ((x >> m & 1) && int(m + sh) < nhi) o |= 1ull << Z.pass.hipos[m + sh];
-        if (j < 64) Z.seg_lo[x] = o >> kLog16; else Z.seg_hi[x] = o >> kLog16;
+        if (j < 64) Z.seg_lo[x] = o >> 1; else Z.seg_hi[x] = o >> 1;
     }
     if (lane == 0) {
         uint64_t base = uint64_t(Z.item.slab) << lo;
@@ -113,22 +109,20 @@ __device__ __forceinline__ void fetch(LeanSlot &Z, const LeanSlot *prev, const B
 // (-1)^{popcount(x & z_t)} = s_t(base) (-1)^{popcount(i & zl_t)} where zl_t is z_t on the slab's local
 // bits, so the slab contributes
 //   sum_t c_t s_t(base) P^(zl_t),   P^(z) = sum_i |a_i|^2 (-1)^{popcount(i & z)},
-// the Walsh-Hadamard transform of the slab's probabilities (state precision).  Element i = tid + NT k: the
+// the Walsh-Hadamard transform of the slab's probabilities (in FP32).  Element i = tid + NT k: the
 // levels over k run in registers, the lane bits by shuffles, the warp bits after one exchange.
-template <typename C, int NT>
-__device__ __forceinline__ double slab_energy(C *sm, int b, const LeanSlot &Z, const BatchTerm *T, uint32_t tid)
+template <int NT>
+__device__ __forceinline__ double slab_energy(float2 *sm, int b, const LeanSlot &Z, const BatchTerm *T, uint32_t tid)
 {
-    using R = decltype(C::x);
-    constexpr int SW = sizeof(C) == 8 ? 1 : 2, TB = NT == 512 ? 9 : 8;
-    constexpr int KB = (sizeof(C) == 8 ? 13 : 12) - TB, K = 1 << KB;
+    constexpr int TB = NT == 512 ? 9 : 8, KB = kMaxBits - TB, K = 1 << KB;
     const uint32_t nsl = 1u << b, lane = tid & 31;
-    R p[K];
+    float p[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const uint32_t i = tid + uint32_t(k) * NT;
-        p[k] = R(0);
+        p[k] = 0.f;
         if (i < nsl) {
-            const C v = sm[swz<SW>(i)];
+            const float2 v = sm[swz<1>(i)];
             p[k] = v.x * v.x + v.y * v.y;
         }
     }
@@ -138,7 +132,7 @@ __device__ __forceinline__ double slab_energy(C *sm, int b, const LeanSlot &Z, c
 #pragma unroll
             for (int k = 0; k < K; ++k)
                 if (!(k >> m & 1)) {
-                    const R u = p[k], w = p[k | 1 << m];
+                    const float u = p[k], w = p[k | 1 << m];
                     p[k] = u + w;
                     p[k | 1 << m] = u - w;
                 }
@@ -148,11 +142,11 @@ __device__ __forceinline__ double slab_energy(C *sm, int b, const LeanSlot &Z, c
         if (j < b) {
 #pragma unroll
             for (int k = 0; k < K; ++k) {
-                const R o = __shfl_xor_sync(0xffffffffu, p[k], 1 << j);
+                const float o = __shfl_xor_sync(0xffffffffu, p[k], 1 << j);
                 p[k] = (lane >> j & 1) ? o - p[k] : p[k] + o;
             }
         }
-    R *pr = reinterpret_cast<R *>(sm);
+    float *pr = reinterpret_cast<float *>(sm);
     __syncthreads();  // every amplitude has been read: the buffer now holds the transform
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -165,16 +159,16 @@ __device__ __forceinline__ double slab_energy(C *sm, int b, const LeanSlot &Z, c
         for (uint32_t q = tid; q < 32u * K; q += NT) {
             const uint32_t i0 = (q & 31) + (q >> 5) * NT;
             if (i0 >= nsl) break;
-            R w[W];
+            float w[W];
 #pragma unroll
-            for (int x = 0; x < W; ++x) w[x] = i0 + 32u * x < nsl ? pr[i0 + 32u * x] : R(0);
+            for (int x = 0; x < W; ++x) w[x] = i0 + 32u * x < nsl ? pr[i0 + 32u * x] : 0.f;
 #pragma unroll
             for (int m = 0; m < WB; ++m)
                 if (5 + m < b) {
 #pragma unroll
                     for (int x = 0; x < W; ++x)
                         if (!(x >> m & 1)) {
-                            const R u = w[x], v = w[x | 1 << m];
+                            const float u = w[x], v = w[x | 1 << m];
                             w[x] = u + v;
                             w[x | 1 << m] = u - v;
                         }
@@ -198,19 +192,17 @@ __device__ __forceinline__ double slab_energy(C *sm, int b, const LeanSlot &Z, c
     return acc;
 }
 
-template <typename R, int RB, int NT, int PER_SM>
+template <int RB, int NT, int PER_SM>
 __global__ void __launch_bounds__(NT, PER_SM)
-    batch_lean_kernel(typename Cx<R>::T *__restrict__ states, const __grid_constant__ BatchArgs a, uint32_t wcap)
+    batch_lean_kernel(float2 *__restrict__ states, const __grid_constant__ BatchArgs a, uint32_t wcap)
 {
-    using C = typename Cx<R>::T;
-    constexpr int SW = sizeof(C) == 8 ? 1 : 2, kLog16 = sizeof(C) == 8 ? 1 : 0;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     LeanShared &S = *reinterpret_cast<LeanShared *>(smem_raw);
     ulonglong2 *const wbufs = reinterpret_cast<ulonglong2 *>(smem_raw + ((sizeof(LeanShared) + 127) & ~size_t(127)));
-    C *const sm = reinterpret_cast<C *>(wbufs + 2 * size_t(wcap));
+    float2 *const sm = reinterpret_cast<float2 *>(wbufs + 2 * size_t(wcap));
     const uint32_t tid = threadIdx.x;
 
-    if (tid < 32) fetch<C>(S.slot[0], nullptr, a, wbufs, wcap, tid);
+    if (tid < 32) fetch(S.slot[0], nullptr, a, wbufs, wcap, tid);
     __syncthreads();
     for (uint32_t k = 0;; k ^= 1u) {
         const LeanSlot &Z = S.slot[k];
@@ -234,14 +226,11 @@ __global__ void __launch_bounds__(NT, PER_SM)
         __syncthreads();
         const bool work = S.late == 0;
         {
-            const int vps_log = Z.pass.lo - kLog16;
-            const uint32_t nvec = 1u << (Z.pass.b - kLog16);
+            const int vps_log = Z.pass.lo - 1;
+            const uint32_t nvec = 1u << (Z.pass.b - 1);
             if (Z.item.pass == 0) {
                 for (uint32_t e = tid; e < (1u << Z.pass.b); e += NT) {
-                    C z;
-                    z.x = (Z.base == 0 && e == 0) ? R(1) : R(0);
-                    z.y = R(0);
-                    sm[swz<SW>(e)] = z;
+                    sm[swz<1>(e)] = make_float2(Z.base == 0 && e == 0 ? 1.f : 0.f, 0.f);
                 }
             } else if (work) {
                 const uint4 *g = reinterpret_cast<const uint4 *>(states + Z.circ.amp_off + Z.base);
@@ -249,11 +238,11 @@ __global__ void __launch_bounds__(NT, PER_SM)
 #pragma unroll 4
                 for (uint32_t v = tid; v < nvec; v += NT) {
                     const uint32_t seg = v >> vps_log, w = v & ((1u << vps_log) - 1);
-                    cp_async16(dst + 16u * chunk_of<C>(v), g + ((Z.seg_lo[seg & 63] | Z.seg_hi[(seg >> 6) & 63]) + w));
+                    cp_async16(dst + 16u * chunk_of(v), g + ((Z.seg_lo[seg & 63] | Z.seg_hi[(seg >> 6) & 63]) + w));
                 }
             }
         }
-        if (tid < 32) fetch<C>(S.slot[k ^ 1u], &Z, a, wbufs + size_t(k ^ 1u) * wcap, wcap, tid);
+        if (tid < 32) fetch(S.slot[k ^ 1u], &Z, a, wbufs + size_t(k ^ 1u) * wcap, wcap, tid);
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
@@ -263,12 +252,12 @@ __global__ void __launch_bounds__(NT, PER_SM)
             uint32_t at = 0;
 #pragma unroll 1
             for (uint32_t o = 0; o < Z.prog.nstages; ++o) {
-                at = run_lean_stage<C, RB>(sm, words, at, static_cast<const C *>(a.pool), Z.base, tid);
+                at = run_lean_stage<float2, RB>(sm, words, at, static_cast<const float2 *>(a.pool), Z.base, tid);
                 __syncthreads();
             }
             if (Z.item.pass == Z.circ.npass - 1) {
                 // the final states are not kept (the batch returns expectation values only)
-                const double part = slab_energy<C, NT>(sm, Z.pass.b, Z, a.terms + Z.circ.term0, tid);
+                const double part = slab_energy<NT>(sm, Z.pass.b, Z, a.terms + Z.circ.term0, tid);
                 if ((tid & 31) == 0) S.red[tid >> 5] = part;
                 __syncthreads();
                 if (tid < 32) {
@@ -278,14 +267,14 @@ __global__ void __launch_bounds__(NT, PER_SM)
                     if (tid == 0) atomicAdd(a.results + Z.item.circ, v);
                 }
             } else {
-                const int vps_log = Z.pass.lo - kLog16;
-                const uint32_t nvec = 1u << (Z.pass.b - kLog16);
+                const int vps_log = Z.pass.lo - 1;
+                const uint32_t nvec = 1u << (Z.pass.b - 1);
                 uint4 *g = reinterpret_cast<uint4 *>(states + Z.circ.amp_off + Z.base);
 #pragma unroll 4
                 for (uint32_t v = tid; v < nvec; v += NT) {
                     const uint32_t seg = v >> vps_log, w = v & ((1u << vps_log) - 1);
                     st_stream(g + ((Z.seg_lo[seg & 63] | Z.seg_hi[(seg >> 6) & 63]) + w),
-                              reinterpret_cast<const uint4 *>(sm)[chunk_of<C>(v)]);
+                              reinterpret_cast<const uint4 *>(sm)[chunk_of(v)]);
                 }
             }
         }
@@ -295,14 +284,13 @@ __global__ void __launch_bounds__(NT, PER_SM)
     }
 }
 
-template <typename R, int RB, int NT, int PER_SM>
+template <int RB, int NT, int PER_SM>
 int launch_t(void *states, const BatchArgs &a, int b_max, void *stream, char *err, size_t errlen)
 {
-    using C = typename Cx<R>::T;
     // longest pass program that is kept in shared memory (longer ones are read from L2)
     const uint32_t wcap = std::min(a.max_words, 1400u);
-    const size_t smem = ((sizeof(LeanShared) + 127) & ~size_t(127)) + 2 * size_t(wcap) * 16 + (sizeof(C) << b_max);
-    auto *const kern = batch_lean_kernel<R, RB, NT, PER_SM>;
+    const size_t smem = ((sizeof(LeanShared) + 127) & ~size_t(127)) + 2 * size_t(wcap) * 16 + (sizeof(float2) << b_max);
+    auto *const kern = batch_lean_kernel<RB, NT, PER_SM>;
     static int attr_dev = -1;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -313,11 +301,11 @@ int launch_t(void *states, const BatchArgs &a, int b_max, void *stream, char *er
     // a second CTA per SM where a round has slabs for it (else it would take work from idle SMs)
     const unsigned sms = unsigned(num_sms()), ctas = a.width > sms ? sms * PER_SM : sms;
     const unsigned grid = std::max(1u, std::min(ctas, unsigned(a.nitems)));
-    if (b_max > (sizeof(C) == 8 ? 13 : 12) || smem > 227 * 1024) {
+    if (b_max > kMaxBits || smem > 227 * 1024) {
         snprintf(err, errlen, "batch slab of %d bits does not fit in shared memory", b_max);
         return QS_EINVAL;
     }
-    kern<<<grid, NT, smem, (cudaStream_t)stream>>>(reinterpret_cast<C *>(states), a, wcap);
+    kern<<<grid, NT, smem, (cudaStream_t)stream>>>(static_cast<float2 *>(states), a, wcap);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         snprintf(err, errlen, "batch launch failed: %s", cudaGetErrorString(e));
@@ -330,8 +318,8 @@ int launch_t(void *states, const BatchArgs &a, int b_max, void *stream, char *er
 
 int launch_batch_lean(int stage_bits, void *states, const BatchArgs &a, int b_max, void *stream, char *err, size_t errlen)
 {
-    if (stage_bits == kStageBitsC64 - 1) return launch_t<float, kStageBitsC64 - 1, 512, 1>(states, a, b_max, stream, err, errlen);
-    return launch_t<float, kStageBitsC64, 256, 2>(states, a, b_max, stream, err, errlen);
+    if (stage_bits == kStageBitsC64 - 1) return launch_t<kStageBitsC64 - 1, 512, 1>(states, a, b_max, stream, err, errlen);
+    return launch_t<kStageBitsC64, 256, 2>(states, a, b_max, stream, err, errlen);
 }
 
 }  // namespace qs
