@@ -440,8 +440,9 @@ struct Builder {
                 break;
             }
             const cd g = M[0] / c, eb = M[2] / (g * s), ed = -M[1] / (g * s);
-            const bool unitary = std::abs(std::abs(eb) - 1.0) <= 1e-12 && std::abs(std::abs(ed) - 1.0) <= 1e-12;
-            if (!unitary || std::abs(M[3] - g * eb * ed * c) > 1e-12 * c || std::abs(c * c + s * s - 1.0) > 1e-12) {
+            const double tol = split_tolerance(plan.dt);
+            const bool unitary = std::abs(std::abs(eb) - 1.0) <= tol && std::abs(std::abs(ed) - 1.0) <= tol;
+            if (!unitary || std::abs(M[3] - g * eb * ed * c) > tol * c || std::abs(c * c + s * s - 1.0) > 1e-12) {
                 bad = true;
                 break;
             }

@@ -570,8 +570,9 @@ uint32_t smem_swizzle(uint32_t i, qs_dtype dt)
 // (all FP64), and write every uncontrolled 1-qubit diagonal diag(d0, d1) as d0 P(arg d1/d0).
 // The real rotation costs half the FMAs of a complex 2x2, and the phases of all qubits between
 // two layers of rotations commute, so the register stages merge them into one table.  The
-// scalar factors g and d0 are collected into one diagonal placed first (a global phase).
-std::vector<CGate> split_one_qubit(const std::vector<CGate> &in)
+// scalar factors g and d0 are collected into one diagonal placed first (a global phase).  Gates off that form by
+// more than rounding (split_tolerance) stay as they were given.
+std::vector<CGate> split_one_qubit(const std::vector<CGate> &in, qs_dtype dt)
 {
     std::vector<CGate> out;
     out.reserve(in.size() * 2);
@@ -594,7 +595,7 @@ std::vector<CGate> split_one_qubit(const std::vector<CGate> &in)
             if (!real && c > 1e-6 && s > 1e-6) {
                 const cd gph = u00 / c;
                 const cd eb = u10 / (gph * s), ed = -u01 / (gph * s);
-                if (std::abs(u11 - gph * eb * ed * c) <= 1e-12) {
+                if (std::abs(u11 - gph * eb * ed * c) <= split_tolerance(dt)) {
                     G *= gph;
                     CGate pd, r, pb;
                     pd.cls = pb.cls = C_DIAG;
@@ -1485,7 +1486,7 @@ int build_plan(const std::vector<CGate> &gates_in, int n, qs_dtype dt, const qs_
         for (const CGate &g : gates) is_tc.push_back(g.cls == C_DENSE && g.tq.size() >= 4);
     } else if (opt.fuse_width > 0) {
         const bool euler = opt.euler != 1;
-        if (opt.blocking && euler) gates = split_one_qubit(gates);
+        if (opt.blocking && euler) gates = split_one_qubit(gates, dt);
         const int kdiag = opt.diag_bits > 0 ? std::min(opt.diag_bits, kMaxDiagBits) : 10;
         int kdense = std::min(opt.fuse_width, kMaxDense);
         if (opt.blocking) kdense = std::min(kdense, lowblock ? b : std::max(1, b - lo));

@@ -85,6 +85,10 @@ double op_cost(const CGate &g, qs_dtype dt);
 void plan_features(const Plan &p, std::vector<float> &rows);
 
 // Default slab and segment bits for a dtype.
+// What a 2x2 matrix may be off its Z-Y-Z form for that form to stand for it: in complex128 a few roundings (the form
+// of a unitary matrix is 1e-15 off), in complex64 less than FP32 shows.
+constexpr double split_tolerance(qs_dtype dt) { return dt == QS_C64 ? 1e-12 : 8e-15; }
+
 int default_slab_bits(qs_dtype dt);
 int default_seg_bits(qs_dtype dt);
 

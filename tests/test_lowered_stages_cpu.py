@@ -146,3 +146,21 @@ def test_batch_circuits_lower_throughout(compare):
             info = qs.qs_plan_info_get(plan)
             qs.qs_plan_destroy(plan)
             assert info["smem_ops"] == 0, (n, slab, width)
+
+
+@pytest.mark.parametrize("form", ["c128", "df"])
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("off", [1e-15, 5e-14, 8e-13])
+def test_nearly_unitary_matrices(compare, off, real, form):
+    """A 2x2 matrix whose last entry is off the unitary one is applied as it is given, however little that is."""
+    opts, tol = FORMS[form]
+    rng = W.SplitMix64(7)
+    gates = []
+    for i in range(40):
+        a, b, c = rng.angle(), 0.0 if real else rng.angle(), 0.0 if real else rng.angle()
+        u = np.array([[math.cos(a), -np.exp(1j * c) * math.sin(a)],
+                      [np.exp(1j * b) * math.sin(a), np.exp(1j * (b + c)) * math.cos(a)]])
+        u[1, 1] *= 1 + off
+        gates.append(Gate("UNITARY", (rng.below(6),), (), (), u))
+    worst, _ = compare(gates, 6, fuse_width=0, **opts)
+    assert worst <= (1e-13 if form == "c128" else tol * 0.1)
