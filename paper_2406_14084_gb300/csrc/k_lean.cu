@@ -3,9 +3,9 @@
 // Same pass as k_slab.cu (load a slab, run its stages, store it), laid out for occupancy instead of
 // a per-CTA pipeline: 256 threads at 128 registers and one slab buffer (64 KiB), so two CTAs share
 // an SM and one computes while the other loads or stores.  Measured with the stage engine, whole
-// circuits: layered-28 complex64 (20 layers, 14 passes) 89.5 -> 41 ms, complete-graph QAOA-23
-// complex64 2.94 -> 0.82 ms, QFT-28 complex128 110 -> 83 ms (FP64 pipe 90 % busy), layered-25
-// complex128 104 -> 96 ms, layered-26 in double-float form 60.9 -> 38.1 ms.
+// circuits, general engine -> now: layered-28 complex64 (20 layers, 14 passes) 89.2 -> 37.9 ms, complete-graph
+// QAOA-23 complex64 2.94 -> 0.53 ms, QFT-28 complex128 110.6 -> 72.1 ms (FP64 pipe 89 % busy), layered-25
+// complex128 104.2 -> 94.7 ms, layered-26 in double-float form 60.9 -> 38.2 ms.
 #include <cuda_runtime.h>
 
 #include <cstdio>

@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(kRedThreads) expect_wht_kernel(const typename 
 // (none where a bin belongs to one warp or CTA).  Bound by HBM (complex64) or the FP64 pipe (complex128,
 // two FMAs per amplitude).  The kernels before added each amplitude into a shared-memory histogram with an
 // FP64 atomic (10 qubits of 27, complex64: 4.73 ms, now 0.19) or kept every bin in registers with one
-// select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.39).  Masks and offsets
+// select and add per bin and amplitude (3 qubits of 28, complex64: 0.62 ms, now 0.36).  Masks and offsets
 // come from the host: small states wait for the chain of dependent instructions, not for memory.
 struct ProbsPlan {
     uint64_t hs;          // selected bits above the low ones

@@ -13,7 +13,7 @@
 //                bits 413 (FMA pipe, about 80 % busy), on one bit 114, table 292-400 (L1 to
 //                registers: 256 B per thread), X 190
 //   complex128   2x2 matrix 1980, table 4330, half table 2170: the FP64 pipe, 2.0 FMA per SM and clock
-//   double-float 2x2 matrix 550 (FMA pipe), table 1030-1130
+//   double-float table 1030-1130 (FMA pipe)
 #pragma once
 
 #include "slab_common.cuh"
