@@ -88,7 +88,8 @@ PAPER_GATES_PER_S = {"qaoa31_c128": 2511 / 17.5, "qft31_c128": 496 / 3.6}
 # per SM per clock (128 FP32, 2 FP64) x 2 flops per FMA.
 ALU_PEAK_TFLOPS = {"c64": 152 * 2.07e9 * 128 * 2 / 1e12, "c128": 152 * 2.07e9 * 2 * 2 / 1e12}
 
-TRAFFIC_SOURCES = ("k_lean.cu", "lean_stage.cuh", "slab_common.cuh", "dev_common.cuh", "df_arith.cuh", "qs_internal.h")
+TRAFFIC_SOURCES = ("k_lean.cuh", "k_lean.cu", "k_lean_c128.cu", "k_lean_df.cu", "lean_stage.cuh", "slab_common.cuh",
+                   "dev_common.cuh", "df_arith.cuh", "qs_internal.h")
 
 
 def slab_kernel_hash() -> str:

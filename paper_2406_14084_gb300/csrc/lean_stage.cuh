@@ -623,7 +623,7 @@ __device__ __forceinline__ void group_addresses(uint32_t (&a)[1 << RB], uint32_t
 }
 
 // A lowered stage is a stream of 16-byte words (format: qs_internal.h).  GlobalWords reads it from
-// device memory; the pass kernel also has a form that carries it in its parameters (k_lean.cu), where
+// device memory; the pass kernel also has a form that carries it in its parameters (k_lean.cuh), where
 // bulk(), used for the factors of tables, still reads device memory.
 //
 // load_word: written as asm so that the two 64-bit halves land in the register pairs that f32x2

@@ -189,7 +189,7 @@ struct PassArgs {
     const void *words;        // device, whole plan: lowered stages (NULL: use the general engine) ...
     const void *pool;         // ... and their conditional tables
 };
-// A pass of lowered register stages only, without a store permutation (k_lean.cu): h_words, its
+// A pass of lowered register stages only, without a store permutation (k_lean.cuh): h_words, its
 // words on the host (nwords of them, nstages stages); d_words, the same on the device.
 struct LeanPassArgs {
     const void *h_words, *d_words, *pool;
