@@ -5,7 +5,7 @@
 // an SM and one computes while the other loads or stores.  Measured with the stage engine, whole
 // circuits, general engine -> now: layered-28 complex64 (20 layers, 14 passes) 89.2 -> 37.9 ms, complete-graph
 // QAOA-23 complex64 2.94 -> 0.53 ms, QFT-28 complex128 110.6 -> 72.1 ms (FP64 pipe 89 % busy), layered-25
-// complex128 104.2 -> 94.7 ms, layered-26 in double-float form 60.9 -> 38.2 ms.
+// complex128 104.2 -> 94.7 ms, layered-26 in double-float form 60.9 -> 37.7 ms.
 //
 // Each arithmetic has a source file of its own (k_lean.cu complex64, k_lean_c128.cu, k_lean_df.cu): a module is
 // loaded whole by the first launch from it, and one with all fifteen kernels grew past the size up to which

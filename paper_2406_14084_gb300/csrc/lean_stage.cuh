@@ -448,29 +448,22 @@ __device__ __forceinline__ void df_prod(const df_factor &a, const dfp &b, unsign
     g = fma2(a.nh, b.l, g);
     g = fma2(a.nl, b.h, g);
 }
-// a b + c as an unnormalised sum h + l, and in normal form
-__device__ __forceinline__ dfp df_fma_sum(const df_factor &a, const dfp &b, const dfp &c)
+// p - g + c, or p - g - c
+template <bool SUB> __device__ __forceinline__ dfp df_sum(unsigned long long p, unsigned long long g, const dfp &c)
 {
-    unsigned long long p, g;
-    df_prod(a, b, p, g);
-    const unsigned long long s = add2(p, c.h), bb = sub2(s, p);
-    return dfp{s, add2(add2(sub2(p, sub2(s, bb)), sub2(c.h, bb)), sub2(c.l, g))};
-}
-__device__ __forceinline__ dfp df_normal(const dfp &u)
-{
+    const unsigned long long s = SUB ? sub2(p, c.h) : add2(p, c.h), bb = sub2(s, p);
+    const unsigned long long e = sub2(p, sub2(s, bb));
+    const unsigned long long t = SUB ? sub2(sub2(e, add2(c.h, bb)), add2(c.l, g)) : add2(add2(e, sub2(c.h, bb)), sub2(c.l, g));
     dfp r;
-    r.h = add2(u.h, u.l);
-    r.l = sub2(u.l, sub2(r.h, u.h));
+    r.h = add2(s, t);
+    r.l = sub2(t, sub2(r.h, s));
     return r;
 }
-__device__ __forceinline__ dfp df_fma(const df_factor &a, const dfp &b, const dfp &c) { return df_normal(df_fma_sum(a, b, c)); }
-// a b - c, the same steps on -c
-__device__ __forceinline__ dfp df_fms(const df_factor &a, const dfp &b, const dfp &c)
+__device__ __forceinline__ dfp df_fma(const df_factor &a, const dfp &b, const dfp &c)
 {
     unsigned long long p, g;
     df_prod(a, b, p, g);
-    const unsigned long long s = sub2(p, c.h), bb = sub2(s, p);
-    return df_normal(dfp{s, sub2(sub2(sub2(p, sub2(s, bb)), add2(c.h, bb)), add2(c.l, g))});
+    return df_sum<false>(p, g, c);
 }
 __device__ __forceinline__ dfp df_mul(const df_factor &a, const dfp &b)
 {
@@ -505,10 +498,14 @@ template <int RB> struct LeanRegs<dfp, RB> {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             if (e & (1 << J)) continue;
-            // (normalised last: the sum is what waits for the other result, no copy of an input)
-            const dfp b = v[e | (1 << J)], u = df_fma_sum(x, b, v[e]);
-            v[e | (1 << J)] = NEG ? df_fms(y, v[e], b) : df_fma(y, v[e], b);
-            v[e] = df_normal(u);
+            // both products before either sum: they hold what the sums need of the old values (26 qubits, 12
+            // layers: 37.7 ms, 38.1 with one result after the other)
+            dfp &a = v[e], &b = v[e | (1 << J)];
+            unsigned long long p, g, q, f;
+            df_prod(x, b, p, g);
+            df_prod(y, a, q, f);
+            a = df_sum<false>(p, g, a);
+            b = df_sum<NEG>(q, f, b);
         }
     }
     static __device__ __forceinline__ float4 factor(ulonglong2 w)
